@@ -72,7 +72,9 @@ enum {
 
 enum { OV_BC_PERIODIC = 0, OV_BC_ANTIPERIODIC = 1, OV_BC_DIRICHLET = 2 };
 
-/* Arithmetic of operator applications. F64: FP64 storage and arithmetic.
+/* Arithmetic of operator applications. F64: FP64 storage and arithmetic; the polynomial recurrences run on
+ * vectors of 57-bit integers with one exponent per site (every number to 2^-56 of the largest of its site;
+ * a NaN or an infinity makes the whole site NaN), which is closer to the exact result than FP64 arithmetic.
  * F32: FP32 storage and arithmetic (reductions accumulate in FP64).
  * F16, BF16: the gauge links and the vectors of the Chebyshev recurrence are stored in 16
  * bits (FP16 with one FP32 scale per site, or BF16) and computed in FP32; the small-space
@@ -142,7 +144,7 @@ typedef struct ov_profile {
     long long clenshaw_regions;  /* loops recorded (one per sign application call) */
     long long clenshaw_launches; /* Wilson-kernel launches inside them */
     double clenshaw_bytes;       /* algorithmic bytes of those launches: per launch and site,
-                                    the 4 links once (576 B FP64; 192 B FP32, two rows stored)
+                                    the 4 links once (576 B F64; 192 B FP32, two rows stored)
                                     plus every input, output and epilogue spinor of each system */
     long long kernel_launches;   /* ov_launch_count() at the time of reading */
 } ov_profile;

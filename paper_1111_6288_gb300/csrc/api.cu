@@ -100,6 +100,8 @@ struct ov_ctx {
     void* U64 = nullptr;
     void* U32 = nullptr;
     void* U16 = nullptr;  // 16-bit links of an FP16 / BF16 context
+    void* Ufx = nullptr;  // fixed-point links of the FP64 recurrences (made from U64 on first use)
+    double fx_scale2 = 0.0;  // squared scale of the operator Ufx holds (0: none yet)
     bool gauge_set = false;
     std::vector<Bank> banks;
     std::vector<DefSpace> dspaces;  // D_ov deflation spaces per (phase, chirality)
@@ -113,6 +115,8 @@ struct ov_ctx {
     double* d_phase = nullptr;  // per-system phases
     signed char* d_chi = nullptr;
     int* d_idx = nullptr;
+    double* d_fxphase = nullptr;  // distinct non-zero phases of a call, and the phase index per system
+    int* d_fxidx = nullptr;
     int cap_sys = 0;
     long long dslash_count = 0;
     long long sign_count = 0;
@@ -178,21 +182,18 @@ constexpr int prec_of() {
                                            : OV_PREC_BF16;
 }
 
-// bytes of one spinor vector, and of one site's spinor and links, per precision
+// bytes of one spinor vector; and of one site's spinor and links in the recurrences of a precision
 size_t vec_bytes(const ov_ctx* c, int prec) {
     if (prec == OV_PREC_F16) return (size_t)half_rhs_bytes<H16>(c->g.V);
     if (prec == OV_PREC_BF16) return (size_t)half_rhs_bytes<B16>(c->g.V);
     return (size_t)12 * c->g.V * (prec == OV_PREC_F64 ? 16 : 8);
 }
-double site_spinor_bytes(int prec) { return prec == OV_PREC_F64 ? 192 : prec == OV_PREC_F32 ? 96 : prec == OV_PREC_F16 ? 52 : 48; }
+double site_spinor_bytes(int prec) { return prec == OV_PREC_F64 ? 196 : prec == OV_PREC_F32 ? 96 : prec == OV_PREC_F16 ? 52 : 48; }
 double site_link_bytes(int prec) { return prec == OV_PREC_F64 ? 576 : prec == OV_PREC_F32 ? 192 : 96; }
 
 
-// Named workspace of at least nvec spinor vectors of the given precision.
-int workspace(ov_ctx* c, const std::string& name, int prec, long long nvec, void** out) {
-    const size_t need = vec_bytes(c, prec) * (size_t)std::max<long long>(nvec, 1);
-    static const char* suffix[4] = {"/64", "/32", "/16", "/b16"};
-    const std::string key = name + suffix[prec];
+// Named workspace of at least `need` bytes.
+int workspace_bytes(ov_ctx* c, const std::string& key, size_t need, void** out) {
     Buf& b = c->ws[key];
     if (b.bytes < need) {
         if (b.ptr) {
@@ -211,6 +212,17 @@ int workspace(ov_ctx* c, const std::string& name, int prec, long long nvec, void
     }
     *out = b.ptr;
     return OV_OK;
+}
+
+// Named workspace of at least nvec spinor vectors of the given precision.
+int workspace(ov_ctx* c, const std::string& name, int prec, long long nvec, void** out) {
+    static const char* suffix[4] = {"/64", "/32", "/16", "/b16"};
+    return workspace_bytes(c, name + suffix[prec], vec_bytes(c, prec) * (size_t)std::max<long long>(nvec, 1), out);
+}
+
+// Named workspace of nvec fixed-point vectors (the FP64 recurrences).
+int workspace_fx(ov_ctx* c, const std::string& name, long long nvec, void** out) {
+    return workspace_bytes(c, name + "/fx", fx_rhs_bytes(c->g.V) * (size_t)std::max<long long>(nvec, 1), out);
 }
 
 // Free the named workspaces whose names start with prefix (after the stream's work is done).
@@ -267,12 +279,16 @@ int ensure_small(ov_ctx* c, long long nmat, long long npartial, int nsys) {
             CK(cudaFree(c->d_chi));
             CK(cudaFree(c->d_idx));
             CK(cudaFree(c->d_red));
+            CK(cudaFree(c->d_fxphase));
+            CK(cudaFree(c->d_fxidx));
         }
         c->cap_sys = std::max(nsys, 64);
         CK(cudaMalloc(&c->d_phase, sizeof(double) * c->cap_sys));
         CK(cudaMalloc(&c->d_chi, c->cap_sys));
         CK(cudaMalloc(&c->d_idx, sizeof(int) * 2 * c->cap_sys));
         CK(cudaMalloc(&c->d_red, sizeof(double2) * c->cap_sys));
+        CK(cudaMalloc(&c->d_fxphase, sizeof(double) * c->cap_sys));
+        CK(cudaMalloc(&c->d_fxidx, sizeof(int) * c->cap_sys));
     }
     return OV_OK;
 }
@@ -394,13 +410,64 @@ bool any_phase(const SysSet& S) {
     return false;
 }
 
+// Links of the FP64 recurrences over the systems of S: the context's fixed-point links of
+// sqrt(scale2) H_w (made from the FP64 links when the scale changes), and for each distinct non-zero
+// phase the x links with that phase.
+int fx_links(ov_ctx* c, const SysSet& S, double scale2, FxLinks* L, cudaStream_t s) {
+    TRY(ensure_small(c, 0, 0, S.n));
+    if (!c->Ufx && cudaMalloc(&c->Ufx, fx_link_bytes(c->g.V)) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, OV_ERR_OOM, "fixed-point gauge field allocation failed");
+    }
+    if (c->fx_scale2 != scale2) {
+        c->fx_scale2 = 0.0;
+        launch_fx_links(c->g, c->p.m0, scale2, c->U64, c->Ufx, s);
+        CKL();
+        c->fx_scale2 = scale2;
+    }
+    L->links = c->Ufx;
+    std::vector<double> ph;
+    std::vector<int> idx(S.n, -1);
+    for (int j = 0; j < S.n; ++j) {
+        if (S.phase[j] == 0.0) continue;
+        size_t q = 0;
+        while (q < ph.size() && ph[q] != S.phase[j]) ++q;
+        if (q == ph.size()) ph.push_back(S.phase[j]);
+        idx[j] = (int)q;
+    }
+    if (ph.empty()) return OV_OK;
+    void* ux;
+    TRY(workspace_bytes(c, "fx_Ux", fx_xlink_bytes(c->g.V) * ph.size(), &ux));
+    CK(cudaMemcpyAsync(c->d_fxphase, ph.data(), sizeof(double) * ph.size(), cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(c->d_fxidx, idx.data(), sizeof(int) * S.n, cudaMemcpyHostToDevice, s));
+    launch_fx_xlinks(c->g, scale2, c->U64, c->Ufx, ux, c->d_fxphase, (int)ph.size(), s);
+    CKL();
+    L->xlinks = ux;
+    L->xidx = c->d_fxidx;
+    return OV_OK;
+}
+
+// The epilogue of a fixed-point application with the same vectors; its links carry the operator's
+// coefficient up to the factor 1/2 of a recurrence's last or first step.
+FxEpilogue fx_epilogue(const Epilogue& e, bool half = false) {
+    FxEpilogue f;
+    f.half = half;
+    f.c1 = e.c1;
+    f.c2 = e.c2;
+    f.c3 = e.c3;
+    f.v1 = e.v1;
+    f.v2 = e.v2;
+    f.v3 = e.v3;
+    return f;
+}
+
 // Launch shape of the Wilson kernel for ns systems of storage type R (right-hand sides per block;
 // for FP32 arithmetic also the 6- or 7-blocks-per-SM register budget and, where the lattice
 // allows, the tiled kernel): timed once on the sign pipeline's own buffers (the Clenshaw-step
 // launch with its epilogue), fastest kept.
-template <typename R>
-int tuned_shape(ov_ctx* c, int ns, const void* U, const double* d_phase, void* in, void* v1, void* v2,
-                void* v3, void* out, cudaStream_t s) {
+// launch(in, out, epilogue, stream, shape) enqueues one application.
+template <typename R, typename F>
+int tuned_shape(ov_ctx* c, int ns, void* in, void* v1, void* v2, void* v3, void* out, cudaStream_t s, F launch) {
     if (c->p.launch_shape > 0) return c->p.launch_shape;  // fixed by the caller
     const auto key = std::make_pair(prec_of<R>(), ns);
     auto it = c->launch_shape.find(key);
@@ -433,9 +500,9 @@ int tuned_shape(ov_ctx* c, int ns, const void* U, const double* d_phase, void* i
         e.v3 = v3;
         char buf[64];
         for (int sh : shapes) {
-            launch_dslash<R>(c->g, c->p.m0, U, in, out, ns, d_phase, e, s, false, sh);  // warm
+            launch(in, out, e, s, sh);  // warm
             cudaEventRecord(e0, s);
-            for (int q = 0; q < 5; ++q) launch_dslash<R>(c->g, c->p.m0, U, in, out, ns, d_phase, e, s, false, sh);
+            for (int q = 0; q < 5; ++q) launch(in, out, e, s, sh);
             cudaEventRecord(e1, s);
             cudaEventSynchronize(e1);
             float ms = 0.f;
@@ -544,6 +611,7 @@ template <typename R, typename ST = R>
 int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogue fin, void* out, cudaStream_t s,
                   int degree = 0) {
     constexpr bool HALF = !std::is_same<R, ST>::value;
+    constexpr bool FX = std::is_same<ST, double>::value;  // the recurrence on fixed-point vectors
     const int prec = prec_of<R>();
     const int precs = prec_of<ST>();
     const int V = c->g.V;
@@ -556,10 +624,18 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
     TRY(workspace(c, "sp_xg", prec, ns, &xg));
     TRY(workspace(c, "sp_xperp", prec, ns, &xperp));
     TRY(workspace(c, "sp_ys", prec, ns, &ys));
-    TRY(workspace(c, "sp_t", precs, ns, &t));
-    TRY(workspace(c, "sp_bA", precs, ns, &bA));
-    TRY(workspace(c, "sp_bB", precs, ns, &bB));
     void *xs = xperp, *p32 = nullptr;  // x_perp in the recurrence's storage; FP32 copy of its result
+    FxLinks fxl;
+    if (FX) {
+        TRY(workspace_fx(c, "sp_t", ns, &t));
+        TRY(workspace_fx(c, "sp_bA", ns, &bA));
+        TRY(workspace_fx(c, "sp_bB", ns, &bB));
+        TRY(workspace_fx(c, "sp_xs", ns, &xs));
+    } else {
+        TRY(workspace(c, "sp_t", precs, ns, &t));
+        TRY(workspace(c, "sp_bA", precs, ns, &bA));
+        TRY(workspace(c, "sp_bB", precs, ns, &bB));
+    }
     if (HALF) {
         TRY(workspace(c, "sp_xs", precs, ns, &xs));
         TRY(workspace(c, "sp_p32", prec, ns, &p32));
@@ -608,15 +684,23 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
     const double m0 = c->p.m0;
     const void* U = links_of<R>(c);
     const void* Us = links_of<ST>(c);
+    if (FX) TRY(fx_links(c, S, alpha, &fxl, s));
     // algorithmic bytes per site of one launch: links once (shared by the systems) plus each
     // system's input, output and epilogue vectors
     const double Vd = (double)V, lb = site_link_bytes(precs), sb = site_spinor_bytes(precs);
     // the whole recurrence (2n launches, no host work) as one stream sequence
     // timing launches read t, bA, x_perp and write bB only (rewritten by the recurrence below)
-    const int rb = tuned_shape<ST>(c, ns, Us, d_phase, t, bA, xs, bA, bB, s);
-    const int nconv = HALF ? 2 : 1;  // launches before the recurrence
+    const int nconv = FX ? 3 : (HALF ? 2 : 1);  // launches besides the recurrence
+    auto step = [&](const void* in, void* o, const Epilogue& e, cudaStream_t st, int shape) {
+        if constexpr (FX) launch_fx_dslash(c->g, fxl, in, o, nullptr, ns, fx_epilogue(e, e.c_op == 0.5 * alpha), st, shape);
+        else launch_dslash<ST>(c->g, m0, Us, in, o, ns, d_phase, e, st, false, shape);
+    };
+    const int rb = tuned_shape<ST>(c, ns, t, bA, xs, bA, bB, s, step);
     auto enqueue = [&](cudaStream_t st) -> void* {
-        if constexpr (HALF) {
+        if constexpr (FX) {
+            launch_fx_from_f64(xperp, xs, V, ns, 1.0, st);
+            launch_fx_from_f64(xperp, bA, V, ns, cf[n], st);
+        } else if constexpr (HALF) {
             launch_to_half<ST>(xperp, xs, V, ns, 1.0, st);
             launch_to_half<ST>(xperp, bA, V, ns, cf[n], st);
         } else {
@@ -626,7 +710,7 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
         void* b2 = nullptr;
         Epilogue plain;
         for (int k = n - 1; k >= 0; --k) {
-            launch_dslash<ST>(c->g, m0, Us, b1, t, ns, d_phase, plain, st, false, rb);
+            step(b1, t, plain, st, rb);
             Epilogue e;
             const double half = (k == 0) ? 0.5 : 1.0;
             e.c_op = alpha * half;
@@ -637,9 +721,13 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
             e.c3 = -1.0;
             e.v3 = b2;
             void* o = b2 ? b2 : bB;
-            launch_dslash<ST>(c->g, m0, Us, t, o, ns, d_phase, e, st, false, rb);
+            step(t, o, e, st, rb);
             b2 = b1;
             b1 = o;
+        }
+        if constexpr (FX) {  // x_perp is not needed any more: its buffer takes P(Q^2) x_perp
+            launch_fx_to_f64(b1, xperp, V, ns, 1.0, st);
+            b1 = xperp;
         }
         return b1;
     };
@@ -656,9 +744,9 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
     }
     void* b1 = nullptr;
     if (c->use_graphs) {
-        char key[256];
-        snprintf(key, sizeof(key), "%d/%d/%d/%d/%p/%p/%p/%p/%p/%p/%p", precs, n, ns, rb, xperp, xs, bA, bB, t,
-                 (const void*)d_phase, Us);
+        char key[384];
+        snprintf(key, sizeof(key), "%d/%d/%d/%d/%p/%p/%p/%p/%p/%p/%p/%p/%p", precs, n, ns, rb, xperp, xs, bA, bB, t,
+                 (const void*)d_phase, FX ? fxl.links : Us, fxl.xlinks, (const void*)fxl.xidx);
         auto it = c->graphs.find(key);
         if (it == c->graphs.end()) {
             if (!c->cap_stream) CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
@@ -908,52 +996,68 @@ int register_bank_internal(ov_ctx* c, double phase, const void* W64, int n, cons
 // Columns of the eigensolver's block per chunk of its filter and residual passes: three vectors of
 // precision prec per column within the context's budget, at least one column.
 int eig_chunk(const ov_ctx* c, int prec, int m) {
-    const long long per_column = 3LL * (long long)vec_bytes(c, prec);
+    const size_t vb = prec == OV_PREC_F64 ? fx_rhs_bytes(c->g.V) : vec_bytes(c, prec);
+    const long long per_column = 3LL * (long long)vb;
     return (int)std::max(1LL, std::min<long long>(m, c->eig_chunk_bytes / per_column));
 }
 
 // Chebyshev filter W <- T_d(Z) W (then normalised by the caller), Z = (2 Q^2 - (1 + a))/(1 - a),
 // which damps the part of the spectrum of Q^2 in [a, 1] and amplifies [0, a).  W: m vectors of
 // precision R, filtered a chunk of columns at a time (the recurrence acts on each column alone;
-// its three temporaries are chunk-sized).
+// its three temporaries are chunk-sized).  FP64: the recurrence runs on fixed-point vectors.
 template <typename R>
-int cheb_filter(ov_ctx* c, void* W, int m, double a, int degree, const double* d_phase, cudaStream_t s) {
+int cheb_filter(ov_ctx* c, void* W, int m, double a, int degree, const SysSet& S, const double* d_phase,
+                cudaStream_t s) {
+    constexpr bool FX = std::is_same<R, double>::value;
     const int prec = prec_of<R>();
     const size_t vb = vec_bytes(c, prec);
     const int cw = eig_chunk(c, prec, m);
     void *Tm, *Tc, *tt;
-    TRY(workspace(c, "flt_Tm", prec, cw, &Tm));
-    TRY(workspace(c, "flt_Tc", prec, cw, &Tc));
-    TRY(workspace(c, "flt_t", prec, cw, &tt));
+    FxLinks fxl;
+    if constexpr (FX) {
+        TRY(workspace_fx(c, "flt_Tm", cw, &Tm));
+        TRY(workspace_fx(c, "flt_Tc", cw, &Tc));
+        TRY(workspace_fx(c, "flt_t", cw, &tt));
+    } else {
+        TRY(workspace(c, "flt_Tm", prec, cw, &Tm));
+        TRY(workspace(c, "flt_Tc", prec, cw, &Tc));
+        TRY(workspace(c, "flt_t", prec, cw, &tt));
+    }
     const double h = c->hw_norm, m0 = c->p.m0;
     const double za = 2.0 / ((1.0 - a) * h * h), zb = -(1.0 + a) / (1.0 - a);
-    const void* U = std::is_same<R, double>::value ? c->U64 : c->U32;
+    if (FX) TRY(fx_links(c, S, 2.0 * za, &fxl, s));
     for (int j0 = 0; j0 < m; j0 += cw) {
         const int nj = std::min(cw, m - j0);
+        auto step = [&](const void* in, void* out, const Epilogue& e) {
+            if constexpr (FX) launch_fx_dslash(c->g, fxl, in, out, nullptr, nj, fx_epilogue(e, e.c_op == za), s, 0);
+            else launch_dslash<R>(c->g, m0, c->U32, in, out, nj, d_phase, e, s);
+        };
         void* Wj = (char*)W + vb * j0;
+        if constexpr (FX) launch_fx_from_f64(Wj, Tm, c->g.V, nj, 1.0, s);  // T_0
+        else CK(cudaMemcpyAsync(Tm, Wj, vb * nj, cudaMemcpyDeviceToDevice, s));
         Epilogue plain;
-        launch_dslash<R>(c->g, m0, U, Wj, tt, nj, d_phase, plain, s);
+        step(Tm, tt, plain);
         Epilogue e1;
         e1.c_op = za;
         e1.c1 = zb;
-        e1.v1 = Wj;
-        launch_dslash<R>(c->g, m0, U, tt, Tc, nj, d_phase, e1, s);  // T_1 = Z W
-        CK(cudaMemcpyAsync(Tm, Wj, vb * nj, cudaMemcpyDeviceToDevice, s));  // T_0
+        e1.v1 = Tm;
+        step(tt, Tc, e1);  // T_1 = Z W
         void* tk = Tc;
         void* tkm = Tm;
         for (int k = 1; k < degree; ++k) {
-            launch_dslash<R>(c->g, m0, U, tk, tt, nj, d_phase, plain, s);
+            step(tk, tt, plain);
             Epilogue e;
             e.c_op = 2.0 * za;
             e.c1 = 2.0 * zb;
             e.v1 = tk;
             e.c3 = -1.0;
             e.v3 = tkm;
-            launch_dslash<R>(c->g, m0, U, tt, tkm, nj, d_phase, e, s);  // T_{k+1} written over T_{k-1}
+            step(tt, tkm, e);  // T_{k+1} written over T_{k-1}
             std::swap(tk, tkm);
         }
+        if constexpr (FX) launch_fx_to_f64(tk, Wj, c->g.V, nj, 1.0, s);
         CKL();
-        CK(cudaMemcpyAsync(Wj, tk, vb * nj, cudaMemcpyDeviceToDevice, s));
+        if constexpr (!FX) CK(cudaMemcpyAsync(Wj, tk, vb * nj, cudaMemcpyDeviceToDevice, s));
     }
     c->dslash_count += 2LL * degree * m;
     return OV_OK;
@@ -1113,7 +1217,8 @@ int ov_destroy(ov_ctx* c) {
             cudaEventDestroy(e.first);
             cudaEventDestroy(e.second);
         }
-    void* ps[] = {c->U64, c->U32, c->U16, c->d_partial, c->d_red, c->d_C, c->d_C2, c->d_phase, c->d_chi, c->d_idx};
+    void* ps[] = {c->U64, c->U32, c->U16, c->Ufx, c->d_partial, c->d_red, c->d_C, c->d_C2, c->d_phase, c->d_chi,
+                  c->d_idx, c->d_fxphase, c->d_fxidx};
     for (void* q : ps)
         if (q) cudaFree(q);
     delete c;
@@ -1229,6 +1334,7 @@ int ov_set_gauge(ov_ctx* c, const void* U, int dtype, ov_stream_t stream) {
         }
     }
     launch_pack_gauge<double>(U, dtype, c->U64, c->g, s);
+    c->fx_scale2 = 0.0;
     launch_pack_gauge<float>(U, dtype, c->U32, c->g, s);
     if (c->p.precision == OV_PREC_F16) launch_pack_gauge_half<H16>(U, dtype, c->U16, c->g.V, s);
     if (c->p.precision == OV_PREC_BF16) launch_pack_gauge_half<B16>(U, dtype, c->U16, c->g.V, s);
@@ -1421,8 +1527,8 @@ static int eigensolve_q_body(ov_ctx* c, double phase, int n_ev, double tol, int 
             const double z0 = (1.0 + a) / (1.0 - a);
             degree = std::max(2, std::min(200, (int)std::ceil(std::acosh(amp) / std::acosh(z0))));
             auto tf = std::chrono::steady_clock::now();
-            if (in_f64) TRY(cheb_filter<double>(c, W, m, a, degree, d_phase, s));
-            else TRY(cheb_filter<float>(c, Wf, m, a, degree, d_phase, s));
+            if (in_f64) TRY(cheb_filter<double>(c, W, m, a, degree, S, d_phase, s));
+            else TRY(cheb_filter<float>(c, Wf, m, a, degree, S, d_phase, s));
             CK(cudaStreamSynchronize(s));
             auto to = std::chrono::steady_clock::now();
             t_filter[in_f64 ? 1 : 0] += std::chrono::duration<double>(to - tf).count();
@@ -2902,73 +3008,59 @@ int prepare_bank_derivative(ov_ctx* c, Bank* b, cudaStream_t s) {
 // and d(Q p) = (dH p + H dp)/h.
 int tangent_poly(ov_ctx* c, const void* X, const SysSet& S, void* Y, cudaStream_t s) {
     const int ns = S.n;
-    const long long n12 = 12LL * c->g.V;
-    const size_t vb = vec_bytes(c, OV_PREC_F64);
-    void *bA, *bB, *dA, *dB, *t, *u, *sv, *r;
-    TRY(workspace(c, "tg_bA", OV_PREC_F64, ns, &bA));
-    TRY(workspace(c, "tg_bB", OV_PREC_F64, ns, &bB));
-    TRY(workspace(c, "tg_dA", OV_PREC_F64, ns, &dA));
-    TRY(workspace(c, "tg_dB", OV_PREC_F64, ns, &dB));
-    TRY(workspace(c, "tg_t", OV_PREC_F64, ns, &t));
-    TRY(workspace(c, "tg_u", OV_PREC_F64, ns, &u));
-    TRY(workspace(c, "tg_s", OV_PREC_F64, ns, &sv));
-    TRY(workspace(c, "tg_r", OV_PREC_F64, ns, &r));
-    TRY(upload_sys(c, S, s));
-    const double* d_phase = any_phase(S) ? c->d_phase : nullptr;
+    void *x, *bA, *bB, *dA, *dB, *t, *u, *sv;
+    TRY(workspace_fx(c, "tg_x", ns, &x));
+    TRY(workspace_fx(c, "tg_bA", ns, &bA));
+    TRY(workspace_fx(c, "tg_bB", ns, &bB));
+    TRY(workspace_fx(c, "tg_dA", ns, &dA));
+    TRY(workspace_fx(c, "tg_dB", ns, &dB));
+    TRY(workspace_fx(c, "tg_t", ns, &t));
+    TRY(workspace_fx(c, "tg_u", ns, &u));
+    TRY(workspace_fx(c, "tg_s", ns, &sv));
     const int n = c->p.poly_degree;
-    const double eps = c->p.eps, h = c->hw_norm, m0 = c->p.m0;
+    const double eps = c->p.eps, h = c->hw_norm;
     const double alpha = 4.0 / ((1.0 - eps) * h * h);
     const double beta = -2.0 * (1.0 + eps) / (1.0 - eps);
-    const void* U = c->U64;
-    launch_scale<double>(c->coeffs[n], X, bA, ns * n12, s);
-    CK(cudaMemsetAsync(dA, 0, vb * ns, s));
+    FxLinks L;  // of g H, g^2 = alpha: t = g H b1, u = g dH b1, s = g (H db1 + dH b1), then u = g dH t
+    TRY(fx_links(c, S, alpha, &L, s));
+    launch_fx_from_f64(X, x, c->g.V, ns, 1.0, s);
+    launch_fx_from_f64(X, bA, c->g.V, ns, c->coeffs[n], s);
+    launch_fx_from_f64(X, dA, c->g.V, ns, 0.0, s);
     void *b1 = bA, *b2 = nullptr, *db1 = dA, *db2 = nullptr;
-    Epilogue plain, derv;
+    FxEpilogue plain, es;
+    es.c1 = 1.0;
+    es.v1 = u;
     for (int k = n - 1; k >= 0; --k) {
-        const double hf = (k == 0) ? 0.5 : 1.0;
-        launch_dslash<double>(c->g, m0, U, b1, t, ns, d_phase, plain, s);          // t = H b1
-        launch_dslash<double>(c->g, m0, U, b1, u, ns, d_phase, derv, s, true);     // u = dH b1
-        Epilogue es;
-        es.c1 = 1.0;
-        es.v1 = u;
-        launch_dslash<double>(c->g, m0, U, db1, sv, ns, d_phase, es, s);           // s = H db1 + u
-        launch_dslash<double>(c->g, m0, U, t, r, ns, d_phase, derv, s, true);      // r = dH t
-        Epilogue eb;
-        eb.c_op = alpha * hf;
-        eb.c1 = beta * hf;
+        launch_fx_dslash(c->g, L, b1, t, u, ns, plain, s);
+        launch_fx_dslash(c->g, L, db1, sv, nullptr, ns, es, s);
+        FxEpilogue eb;
+        eb.half = k == 0;
+        eb.c1 = eb.half ? 0.5 * beta : beta;
         eb.v1 = b1;
         eb.c2 = c->coeffs[k];
-        eb.v2 = X;
+        eb.v2 = x;
         eb.c3 = -1.0;
         eb.v3 = b2;
         void* ob = b2 ? b2 : bB;
-        launch_dslash<double>(c->g, m0, U, t, ob, ns, d_phase, eb, s);             // b_k
-        Epilogue ed;
-        ed.c_op = alpha * hf;
-        ed.c1 = beta * hf;
+        launch_fx_dslash(c->g, L, t, ob, u, ns, eb, s);  // b_k
+        FxEpilogue ed = eb;
         ed.v1 = db1;
-        ed.c2 = alpha * hf;
-        ed.v2 = r;
-        ed.c3 = -1.0;
+        ed.c2 = eb.half ? 0.5 : 1.0;
+        ed.v2 = u;
         ed.v3 = db2;
         void* od = db2 ? db2 : dB;
-        launch_dslash<double>(c->g, m0, U, sv, od, ns, d_phase, ed, s);            // db_k
+        launch_fx_dslash(c->g, L, sv, od, nullptr, ns, ed, s);  // db_k
         b2 = b1;
         b1 = ob;
         db2 = db1;
         db1 = od;
     }
     CKL();
-    c->dslash_count += 6LL * n * ns;
+    c->dslash_count += 4LL * n * ns;
     // Y = (H dp + dH p)/h with p = b1, dp = db1
-    Epilogue ep;
-    ep.c_op = 1.0 / h;
-    launch_dslash<double>(c->g, m0, U, b1, t, ns, d_phase, ep, s, true);           // t = dH p / h
-    Epilogue ey;
-    ey.c_op = 1.0 / h;
-    ey.c1 = 1.0;
-    ey.v1 = t;
-    launch_dslash<double>(c->g, m0, U, db1, Y, ns, d_phase, ey, s);
+    launch_fx_dslash(c->g, L, b1, t, u, ns, plain, s);
+    launch_fx_dslash(c->g, L, db1, sv, nullptr, ns, es, s);
+    launch_fx_to_f64(sv, Y, c->g.V, ns, 1.0 / (h * std::sqrt(alpha)), s);
     CKL();
     return OV_OK;
 }

@@ -84,6 +84,38 @@ void launch_dslash(const Geom& g, double m0, const void* links, const void* in, 
                    const double* d_phase, const Epilogue& e, cudaStream_t s, bool deriv = false,
                    int shape = 0);
 
+// ---- kernels: fx.cu ---------------------------------------------------------
+// FP64 recurrences on site-scaled fixed-point vectors (fx_arith.h).  A vector of one right-hand side
+// takes fx_rhs_bytes(V) bytes; the links (from the FP64 links, boundary signs folded in) fx_link_bytes(V),
+// and the x links of one field phase fx_xlink_bytes(V).
+struct FxLinks {
+    const void* links = nullptr;
+    const void* xlinks = nullptr;  // [phase] x links with the phase folded in
+    const int* xidx = nullptr;     // device [nrhs]: phase index of each system, -1 for none (null: no field)
+};
+// out = (1/2 if half) g H_w in + c1 v1 + c2 v2 + c3 v3; v3 may be out.
+struct FxEpilogue {
+    bool half = false;
+    double c1 = 0.0, c2 = 0.0, c3 = 0.0;
+    const void* v1 = nullptr;
+    const void* v2 = nullptr;
+    const void* v3 = nullptr;
+};
+size_t fx_rhs_bytes(int V);
+size_t fx_link_bytes(int V);
+size_t fx_xlink_bytes(int V);
+// Links of g H_w, g = sqrt(scale2).
+void launch_fx_links(const Geom& g, double m0, double scale2, const void* U64, void* dst, cudaStream_t s);
+void launch_fx_xlinks(const Geom& g, double scale2, const void* U64, const void* links, void* dst,
+                      const double* d_phases, int nphase, cudaStream_t s);
+// FP64 spinors (internal layout) times factor -> fixed point, and back (times factor).
+void launch_fx_from_f64(const void* in, void* out, int V, int nrhs, double factor, cudaStream_t s);
+void launch_fx_to_f64(const void* in, void* out, int V, int nrhs, double factor, cudaStream_t s);
+// One application on fixed-point vectors.  out_deriv (may be null): g dH_w/dphi in, without the
+// epilogue.  shape: right-hand sides per thread block in the low bits (0: default).
+void launch_fx_dslash(const Geom& g, const FxLinks& U, const void* in, void* out, void* out_deriv, int nrhs,
+                      const FxEpilogue& e, cudaStream_t s, int shape = 0);
+
 // ---- kernels: blas.cu -----------------------------------------------------
 // ABI spinor [rhs][site][12] (dtype_in: 0 complex128, 1 complex64) -> internal [rhs][12][V] of R.
 template <typename R>
