@@ -841,32 +841,36 @@ int apply_generic(ov_ctx* c, const void* in, void* out, int nrhs, const double* 
                   cudaStream_t s) {
     const int prec = prec_of<R>();
     const int dt = (prec == OV_PREC_F64) ? OV_C128 : OV_C64;
+    SysSet S = make_sys(nrhs, phase);
+    TRY(phase_check(c, S));
+    if (kind == 0 || kind == 1) {  // D_w (0) or H_w (1), kind 0 with gamma5 H_w = D_w
+        const double* d_phase = nullptr;
+        if (any_phase(S)) {
+            TRY(upload_sys(c, S, s));
+            d_phase = c->d_phase;
+        }
+        // FP64 reads the caller's array in place, or a copy where the two arrays overlap
+        const void* X = in;
+        const size_t bytes = vec_bytes(c, prec) * nrhs;
+        const bool overlap = (const char*)in < (const char*)out + bytes && (const char*)out < (const char*)in + bytes;
+        if (prec != OV_PREC_F64 || overlap) {
+            void* q;
+            TRY(workspace(c, "io_in", prec_of<ST>(), nrhs, &q));
+            if (prec == OV_PREC_F64) CK(cudaMemcpyAsync(q, in, bytes, cudaMemcpyDeviceToDevice, s));
+            else launch_pack_spinor<ST>(in, dt, q, c->g.V, nrhs, s);
+            X = q;
+        }
+        launch_wilson_abi<ST>(c->g, c->p.m0, links_of<ST>(c), X, out, nrhs, d_phase, kind == 0, s, c->p.launch_shape);
+        CKL();
+        c->dslash_count += nrhs;
+        return OV_OK;
+    }
     void *X, *Y;
     TRY(workspace(c, "io_in", prec, nrhs, &X));
     TRY(workspace(c, "io_out", prec, nrhs, &Y));
     launch_pack_spinor<R>(in, dt, X, c->g.V, nrhs, s);
     CKL();
-    SysSet S = make_sys(nrhs, phase);
-    TRY(phase_check(c, S));
-    if (kind == 0 || kind == 1) {  // D_w (0) or H_w (1)
-        TRY(upload_sys(c, S, s));
-        Epilogue e;
-        e.g5 = (kind == 0);  // gamma5 H_w = D_w
-        const double* d_phase = any_phase(S) ? c->d_phase : nullptr;
-        const int shape = c->p.launch_shape;  // 0: the default shape
-        if constexpr (std::is_same<R, ST>::value) {
-            launch_dslash<R>(c->g, c->p.m0, links_of<R>(c), X, Y, nrhs, d_phase, e, s, false, shape);
-        } else {  // input rounded to the 16-bit format, output read back into FP32
-            void *Xh, *Yh;
-            TRY(workspace(c, "io_in", prec_of<ST>(), nrhs, &Xh));
-            TRY(workspace(c, "io_out", prec_of<ST>(), nrhs, &Yh));
-            launch_to_half<ST>(X, Xh, c->g.V, nrhs, 1.0, s);
-            launch_dslash<ST>(c->g, c->p.m0, links_of<ST>(c), Xh, Yh, nrhs, d_phase, e, s, false, shape);
-            launch_from_half<ST>(Yh, Y, c->g.V, nrhs, s);
-        }
-        CKL();
-        c->dslash_count += nrhs;
-    } else if (kind == 2) {  // sign
+    if (kind == 2) {  // sign
         Epilogue fin;
         fin.c_op = 1.0 / c->hw_norm;
         fin.c1 = 1.0;

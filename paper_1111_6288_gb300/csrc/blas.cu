@@ -90,36 +90,51 @@ template <> struct SiteIO<float> {
 
 // ---- packing -------------------------------------------------------------
 
-template <typename TI, typename R>
-__global__ void pack_spinor_k(const TI* __restrict__ abi, void* __restrict__ out, int V, int nrhs) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)V * nrhs) return;
-    const int r = (int)(idx / V), s = (int)(idx % V);
-    const TI* src = abi + ((long long)r * V + s) * 12;
-    typename SiteIO<R>::T p[12];
+// The caller's arrays hold a site's 12 numbers together, the internal planes one number of consecutive
+// sites: a block turns 128 sites of one right-hand side (blockIdx.y) around in shared memory (rows of 13,
+// free of bank conflicts), so that both sides are read and written in full lines.
+constexpr int PT = 128;
+
+template <typename TI, typename ST>
+__global__ void __launch_bounds__(PT) pack_spinor_k(const TI* __restrict__ abi, void* __restrict__ out, int V) {
+    __shared__ TI sh[PT * 13];
+    const int s0 = blockIdx.x * PT, ns = min(PT, V - s0), t = threadIdx.x;
+    const TI* src = abi + ((long long)blockIdx.y * V + s0) * 12;
+    for (int i = t; i < ns * 12; i += PT) sh[i / 12 * 13 + i % 12] = src[i];
+    __syncthreads();
+    if (t >= ns) return;
+    if constexpr (std::is_same<ST, double>::value || std::is_same<ST, float>::value) {
+        typename SiteIO<ST>::T p[12];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        p[k].x = (R)src[k].x;
-        p[k].y = (R)src[k].y;
+        for (int k = 0; k < 12; ++k) {
+            p[k].x = (ST)sh[t * 13 + k].x;
+            p[k].y = (ST)sh[t * 13 + k].y;
+        }
+        SiteIO<ST>::store((char*)out + (long long)blockIdx.y * 12 * V * sizeof(p[0]), V, s0 + t, p);
+    } else {  // rounded to 16-bit storage
+        float2 p[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) p[k] = make_float2((float)sh[t * 13 + k].x, (float)sh[t * 13 + k].y);
+        half_store_site<ST>((char*)out + blockIdx.y * half_rhs_bytes<ST>(V), V, s0 + t, p);
     }
-    SiteIO<R>::store((char*)out + (long long)r * 12 * V * sizeof(typename SiteIO<R>::T), V, s, p);
 }
 
 template <typename R, typename TO>
-__global__ void unpack_spinor_k(const void* __restrict__ in, TO* __restrict__ abi, int V, int nrhs) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)V * nrhs) return;
-    const int r = (int)(idx / V), s = (int)(idx % V);
-    typename SiteIO<R>::T p[12];
-    SiteIO<R>::load((const char*)in + (long long)r * 12 * V * sizeof(typename SiteIO<R>::T), V, s, p);
-    TO* dst = abi + ((long long)r * V + s) * 12;
+__global__ void __launch_bounds__(PT) unpack_spinor_k(const void* __restrict__ in, TO* __restrict__ abi, int V) {
+    __shared__ TO sh[PT * 13];
+    const int s0 = blockIdx.x * PT, ns = min(PT, V - s0), t = threadIdx.x;
+    if (t < ns) {
+        typename SiteIO<R>::T p[12];
+        SiteIO<R>::load((const char*)in + (long long)blockIdx.y * 12 * V * sizeof(p[0]), V, s0 + t, p);
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        TO o;
-        o.x = p[k].x;
-        o.y = p[k].y;
-        dst[k] = o;
+        for (int k = 0; k < 12; ++k) {
+            sh[t * 13 + k].x = p[k].x;
+            sh[t * 13 + k].y = p[k].y;
+        }
     }
+    __syncthreads();
+    TO* dst = abi + ((long long)blockIdx.y * V + s0) * 12;
+    for (int i = t; i < ns * 12; i += PT) dst[i] = sh[i / 12 * 13 + i % 12];
 }
 
 // FP64 links: 9 planes of double2 per direction, the link U_mu(n) on the last slice of
@@ -570,23 +585,19 @@ inline int grid_for(long long n, int bs, int cap = 152 * 16) {
 
 template <typename R>
 void launch_pack_spinor(const void* abi, int dtype_in, void* internal, int V, int nrhs, cudaStream_t s) {
-    const long long n = (long long)V * nrhs;
-    const int g = (int)((n + 255) / 256);
-    if (dtype_in == 0)
-        pack_spinor_k<double2, R><<<g, 256, 0, s>>>((const double2*)abi, internal, V, nrhs);
-    else
-        pack_spinor_k<float2, R><<<g, 256, 0, s>>>((const float2*)abi, internal, V, nrhs);
+    const dim3 grid((V + PT - 1) / PT, nrhs);
+    if (dtype_in == 0) pack_spinor_k<double2, R><<<grid, PT, 0, s>>>((const double2*)abi, internal, V);
+    else pack_spinor_k<float2, R><<<grid, PT, 0, s>>>((const float2*)abi, internal, V);
     count_launch();
 }
+template void launch_pack_spinor<H16>(const void*, int, void*, int, int, cudaStream_t);
+template void launch_pack_spinor<B16>(const void*, int, void*, int, int, cudaStream_t);
 
 template <typename R>
 void launch_unpack_spinor(const void* internal, void* abi, int dtype_out, int V, int nrhs, cudaStream_t s) {
-    const long long n = (long long)V * nrhs;
-    const int g = (int)((n + 255) / 256);
-    if (dtype_out == 0)
-        unpack_spinor_k<R, double2><<<g, 256, 0, s>>>(internal, (double2*)abi, V, nrhs);
-    else
-        unpack_spinor_k<R, float2><<<g, 256, 0, s>>>(internal, (float2*)abi, V, nrhs);
+    const dim3 grid((V + PT - 1) / PT, nrhs);
+    if (dtype_out == 0) unpack_spinor_k<R, double2><<<grid, PT, 0, s>>>(internal, (double2*)abi, V);
+    else unpack_spinor_k<R, float2><<<grid, PT, 0, s>>>(internal, (float2*)abi, V);
     count_launch();
 }
 

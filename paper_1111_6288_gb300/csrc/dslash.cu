@@ -410,17 +410,17 @@ __device__ __forceinline__ Cx<R> field_phase(const Args<R>& a, int r, int t) {
 }
 
 // The epilogue: z = c_op gamma5 (diag psi - acc / 2) (DERIV: c_op gamma5 (-acc / 2)), + c1 v1,
-// gamma5, chiral projection, + c2 v2 + c3 v3, stored at site s of right-hand side r.
+// gamma5, chiral projection, + c2 v2 + c3 v3, of site s of right-hand side r.
 template <typename ST, bool DERIV, typename R = typename Arith<ST>::type>
-__device__ __forceinline__ void finish(const Args<R>& a, int s, int r, const Cx<R> (&psi)[12],
-                                       const Cx<R> (&acc)[12]) {
+__device__ __forceinline__ void epilogue(const Args<R>& a, int s, int r, const Cx<R> (&psi)[12],
+                                         const Cx<R> (&acc)[12], Cx<R> (&z)[12]) {
     const long long V = a.V;
     const long long off = (long long)r * IO<ST>::rhs_bytes(V);  // bytes per right-hand side
     const R cop = a.c_op, c1 = a.c1;
     const R c2 = a.c2r ? a.c2 * (R)a.c2r[(long long)r * a.c2r_stride] : a.c2;
     // cd psi + ch acc on the upper spins, negated on the lower
     const R cd = cop * a.diag, ch = R(-0.5) * cop;
-    Cx<R> z[12], tmp[12];
+    Cx<R> tmp[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
         const R sd = k < 6 ? cd : -cd, sh = k < 6 ? ch : -ch;
@@ -460,7 +460,13 @@ __device__ __forceinline__ void finish(const Args<R>& a, int s, int r, const Cx<
 #pragma unroll
         for (int k = 0; k < 12; ++k) z[k] = cadd(z[k], cscale(a.c3, tmp[k]));
     }
-    IO<ST>::store((char*)a.out + off, V, s, z);
+}
+template <typename ST, bool DERIV, typename R = typename Arith<ST>::type>
+__device__ __forceinline__ void finish(const Args<R>& a, int s, int r, const Cx<R> (&psi)[12],
+                                       const Cx<R> (&acc)[12]) {
+    Cx<R> z[12];
+    epilogue<ST, DERIV>(a, s, r, psi, acc, z);
+    IO<ST>::store((char*)a.out + (long long)r * IO<ST>::rhs_bytes(a.V), a.V, s, z);
 }
 
 // ---- bulk copies into shared memory (TMA, one dimension) and their barrier ----
@@ -533,6 +539,13 @@ __global__ void bounded_wait_selftest_k(long long limit) {
 
 constexpr int DSLASH_THREADS = OVL_DSLASH_THREADS;
 
+// FP64 applications that take the eight-lanes-a-site kernel: up to 16384 sites (thread a site against
+// eight lanes, one vector / twelve: 37 / 37 us against 10.4 / 10.5 us on 4^4, 37 / 193 against 21 / 170 us on
+// 8^3 x 16, 37 / 350 against 33 / 333 us on 16384 sites; equal at 16^3 x 32); with a field, whose phase every
+// lane then works out and applies, up to 8192 sites and vectors together (41 against 24 us on one 8^4 vector,
+// 109 against 129 us on twelve).
+__host__ inline bool split_sites(long long V, int nrhs, bool field) { return field ? V * nrhs <= 8192 : V <= 16384; }
+
 // Blocks per SM that the register allocation must allow.  FP32: 6 (80 registers, no
 // spills), 7-9 % faster than the unconstrained 87 registers at 16^3 x 32 and 24^3 x 48,
 // where more resident warps hide the latency of the neighbour loads; FP64 needs its
@@ -591,6 +604,198 @@ __global__ void __launch_bounds__(DSLASH_THREADS, MINB) dslash_kernel(Args<typen
         src.load(s, 0, psi);
     }
     finish<ST, DERIV>(a, s, r, psi, acc);
+}
+
+// ---- single applications on the caller's arrays ([rhs][site][12] complex) --------------------
+
+// Neighbour spinors read from the caller's array.
+struct AbiSrc {
+    const double2* in;
+    __device__ __forceinline__ void load(int site, int, Cx<double> (&p)[12]) const {
+        const double2* b = in + (long long)site * 12;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const double2 v = __ldg(b + k);
+            p[k] = {v.x, v.y};
+        }
+    }
+};
+
+// A site's numbers as 16-bit storage keeps them.
+template <typename S>
+__device__ __forceinline__ void round_site(Cx<float> (&z)[12]) {
+    if constexpr (!std::is_same<S, float>::value && !std::is_same<S, double>::value) {
+        float scale = 1.0f, inv = 1.0f;
+        if constexpr (HalfSpinor<S>::scaled) {
+            float m = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 12; ++k) m = fmaxf(m, fmaxf(fabsf(z[k].re), fabsf(z[k].im)));
+            if (m > 0.0f) m = fmaxf(m, 1e-30f);
+            scale = m;
+            inv = m > 0.0f ? 1.0f / m : 0.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            float2 v = half_word<S>(half_pack<S>(z[k].re * inv, z[k].im * inv));
+            if constexpr (HalfSpinor<S>::scaled) v = make_float2(v.x * scale, v.y * scale);
+            z[k] = {v.x, v.y};
+        }
+    }
+}
+
+// One application written straight to the caller's array, turned around in shared memory so that full
+// lines are written; FP64 also reads the caller's array in place (its neighbour loads, which then touch a
+// line each, hide behind the FP64 pipe), FP32 and 16-bit applications read the internal planes.  Against
+// pack, stencil and unpack this saves the unpacking pass (FP64: both; 16 bits: also the passes through
+// FP32): 12 vectors of 24^3 x 48 with a field in FP32 1224 -> 894 us, one FP64 vector of 16^3 x 32 257 ->
+// 229 us, 12 BF16 vectors 330 -> 180 us.
+template <typename ST, int MINB>
+__global__ void __launch_bounds__(DSLASH_THREADS, MINB) wilson_abi_kernel(Args<typename Arith<ST>::type> a, int nrhs) {
+    using R = typename Arith<ST>::type;
+    constexpr bool F64 = std::is_same<ST, double>::value;
+    typedef typename C2<R>::T T2;
+    __shared__ T2 sh[DSLASH_THREADS * 13];
+    const int s0 = blockIdx.x * blockDim.x, s = s0 + threadIdx.x;
+    const int r = blockIdx.y * blockDim.y + threadIdx.y;
+    const long long V = a.V;
+    T2* row = sh + (threadIdx.y * blockDim.x + threadIdx.x) * 13;
+    if (s < V && r < nrhs) {
+        int t = s;
+        const int x0 = t % a.L[0];
+        t /= a.L[0];
+        const int x1 = t % a.L[1];
+        t /= a.L[1];
+        const int x2 = t % a.L[2];
+        const int x3 = t / a.L[2];
+        const Cx<R> ph = field_phase(a, r, x3);
+        Cx<R> acc[12], psi[12], z[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k] = {R(0), R(0)};
+        auto hops = [&](const auto& src) {
+            both_hops<ST, 2, false>(a, src, s, x2, 0, 0, ph, acc);
+            both_hops<ST, 3, false>(a, src, s, x3, 0, 0, ph, acc);
+            if (a.phase) both_hops<ST, 0, true>(a, src, s, x0, 0, 0, ph, acc);
+            else both_hops<ST, 0, false>(a, src, s, x0, 0, 0, ph, acc);
+            both_hops<ST, 1, false>(a, src, s, x1, 0, 0, ph, acc);
+            src.load(s, 0, psi);
+        };
+        if constexpr (F64) hops(AbiSrc{(const double2*)a.in + (long long)r * 12 * V});
+        else hops(GlobalSrc<ST>{(const char*)a.in + (long long)r * IO<ST>::rhs_bytes(V), V});
+        epilogue<ST, false>(a, s, r, psi, acc, z);
+        if constexpr (!F64) round_site<ST>(z);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            row[k].x = z[k].re;
+            row[k].y = z[k].im;
+        }
+    }
+    __syncthreads();
+    if (r >= nrhs) return;
+    const int n = min((int)blockDim.x, (int)(V - s0)) * 12;
+    T2* out = (T2*)a.out + ((long long)r * V + s0) * 12;
+    const T2* mine = sh + threadIdx.y * blockDim.x * 13;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = mine[i / 12 * 13 + i % 12];
+}
+
+// i^code z, code a runtime value: a swap and two sign bits, no arithmetic.
+__device__ __forceinline__ double with_sign(double v, bool neg) {
+    return __longlong_as_double(__double_as_longlong(v) ^ ((long long)neg << 63));
+}
+__device__ __forceinline__ Cx<double> mulu_rt(int code, Cx<double> z) {
+    const double re = (code & 1) ? z.im : z.re, im = (code & 1) ? z.re : z.im;
+    return {with_sign(re, code == 1 || code == 2), with_sign(im, code >= 2)};
+}
+
+// The same on a lattice of few sites, eight lanes a site, one hop each.  One thread a site leaves most SMs
+// idle there, and an SM's FP64 pipe takes 16 cycles for a warp's instruction, 909 of them a site: 4^4 takes
+// 30 us on two SMs (8 us on eight, in blocks of one warp).  Here a warp holds four sites; the lanes' sums are
+// exchanged so that lane l ends with numbers 3 l .. 3 l + 2 of its site's 24.  Hops differ between lanes
+// only in addresses and in the units i^k, which are applied as swaps and sign bits.
+__global__ void __launch_bounds__(32) wilson_split_kernel(Args<double> a, int nrhs) {
+    const int lane = threadIdx.x, l = lane & 7, r = blockIdx.y;
+    const long long V = a.V;
+    const int site = blockIdx.x * 4 + (lane >> 3), s = min(site, (int)V - 1);
+    const int mu = l >> 1;
+    const bool fwd = (l & 1) == 0;
+    int x[4], t = s;
+    x[0] = t % a.L[0];
+    t /= a.L[0];
+    x[1] = t % a.L[1];
+    t /= a.L[1];
+    x[2] = t % a.L[2];
+    x[3] = t / a.L[2];
+    const int xm = mu == 0 ? x[0] : mu == 1 ? x[1] : mu == 2 ? x[2] : x[3];
+    const int L = mu == 0 ? a.L[0] : mu == 1 ? a.L[1] : mu == 2 ? a.L[2] : a.L[3];
+    const int st = mu == 0 ? a.stride[0] : mu == 1 ? a.stride[1] : mu == 2 ? a.stride[2] : a.stride[3];
+    const double bc = mu == 0 ? a.bcf[0] : mu == 1 ? a.bcf[1] : mu == 2 ? a.bcf[2] : a.bcf[3];
+    const bool edge = fwd ? xm == L - 1 : xm == 0;
+    const int nb = fwd ? (edge ? s - (L - 1) * st : s + st) : (edge ? s + (L - 1) * st : s - st);
+    const bool none = edge && bc == 0.0;  // Dirichlet
+    // G of mu: i^A, i^B on the diagonal (z, t) or off it (x, y)
+    const int A = mu == 0 ? 3 : mu == 1 ? 2 : mu == 2 ? 3 : 0, B = mu == 0 ? 3 : mu == 1 ? 0 : mu == 2 ? 1 : 0;
+    const bool diag = mu >= 2;
+    const int S = fwd ? 2 : 0;
+    const double2* in = (const double2*)a.in + (long long)r * 12 * V;
+    const double2* p = in + (long long)nb * 12;
+    const double2* ul = (const double2*)a.U + (long long)mu * 9 * V + (fwd ? s : nb);
+    Cx<double> h[2][3], w[2][3];
+    auto ld = [](const double2* q) {
+        const double2 v = __ldg(q);
+        return Cx<double>{v.x, v.y};
+    };
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        h[0][c] = cadd(ld(p + c), mulu_rt((A + S) & 3, ld(p + (diag ? 6 : 9) + c)));
+        h[1][c] = cadd(ld(p + 3 + c), mulu_rt((B + S) & 3, ld(p + (diag ? 9 : 6) + c)));
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            Cx<double> u = ld(ul + (long long)(fwd ? 3 * i + j : 3 * j + i) * V);
+            u.im = with_sign(u.im, !fwd);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) w[q][i] = j == 0 ? cmul(u, h[q][0]) : cfma(u, h[q][j], w[q][i]);
+        }
+    if (a.phase) {
+        double sn, cs;
+        sincos(a.phase[r] * (double)x[3], &sn, &cs);
+        const Cx<double> f = mu == 0 ? Cx<double>{cs, fwd ? sn : -sn} : Cx<double>{1.0, 0.0};
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) w[q][i] = cmul(f, w[q][i]);
+    }
+    double v[24];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const Cx<double> l0 = mulu_rt((4 - A + S) & 3, w[0][i]), l1 = mulu_rt((4 - B + S) & 3, w[1][i]);
+        const Cx<double> z[4] = {w[0][i], w[1][i], diag ? l0 : l1, diag ? l1 : l0};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            v[2 * (3 * q + i)] = none ? 0.0 : z[q].re;
+            v[2 * (3 * q + i) + 1] = none ? 0.0 : z[q].im;
+        }
+    }
+    // lanes of a site add up: halves, quarters, eighths of the 24 numbers
+#pragma unroll
+    for (int half = 12; half >= 3; half /= 2) {
+        const int m = half == 12 ? 4 : half == 6 ? 2 : 1;
+        const bool up = (l & m) != 0;
+#pragma unroll
+        for (int k = 0; k < 12; ++k)
+            if (k < half) {
+                const double keep = up ? v[half + k] : v[k], send = up ? v[k] : v[half + k];
+                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+            }
+    }
+    if (site >= V) return;
+    const bool lower = l >= 4;  // numbers 12 .. 23: spins 2 and 3
+    const double sg = lower && !a.g5 ? -a.c_op : a.c_op;
+    const double* own = (const double*)in + (long long)s * 24 + 3 * l;
+    double* out = (double*)a.out + ((long long)r * V + s) * 24 + 3 * l;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) out[k] = fmar(sg * a.diag, __ldg(own + k), (-0.5 * sg) * v[k]);
 }
 
 // Tiled H_w: a block covers `rows` whole x-rows of one (z, t) slice (blockDim.x = rows * Lx
@@ -698,10 +903,10 @@ int take_wait_timeouts() {
     return v;
 }
 
-template <typename S>
-void launch_dslash(const Geom& g, double m0, const void* links, const void* in, void* out, int nrhs,
-                   const double* d_phase, const Epilogue& e, cudaStream_t s, bool deriv, int shape) {
-    using R = typename Arith<S>::type;
+namespace {
+template <typename S, typename R = typename Arith<S>::type>
+Args<R> make_args(const Geom& g, double m0, const void* links, const void* in, void* out, const double* d_phase,
+                  const Epilogue& e) {
     Args<R> a;
     a.U = links;
     a.in = in;
@@ -727,6 +932,44 @@ void launch_dslash(const Geom& g, double m0, const void* links, const void* in, 
     }
     a.V = g.V;
     a.g5 = e.g5;
+    return a;
+}
+}  // namespace
+
+template <typename S>
+void launch_wilson_abi(const Geom& g, double m0, const void* links, const void* in, void* out, int nrhs,
+                       const double* d_phase, bool g5, cudaStream_t s, int shape) {
+    Epilogue e;
+    e.g5 = g5;
+    const auto a = make_args<S>(g, m0, links, in, out, d_phase, e);
+    if constexpr (std::is_same<S, double>::value) {
+        if (split_sites(g.V, nrhs, d_phase != nullptr)) {
+            wilson_split_kernel<<<dim3((g.V + 3) / 4, nrhs), 32, 0, s>>>(a, nrhs);
+            count_launch();
+            return;
+        }
+    }
+    int by = (shape & kShapeRhsMask) > 0 ? (shape & kShapeRhsMask) : (nrhs > 1 ? 2 : 1);
+    while (by > 1 && by > nrhs) by >>= 1;
+    const int bx = DSLASH_THREADS / by;
+    const dim3 block(bx, by), grid((g.V + bx - 1) / bx, (nrhs + by - 1) / by);
+    wilson_abi_kernel<S, MinBlocks<S>::value><<<grid, block, 0, s>>>(a, nrhs);
+    count_launch();
+}
+template void launch_wilson_abi<double>(const Geom&, double, const void*, const void*, void*, int, const double*, bool,
+                                        cudaStream_t, int);
+template void launch_wilson_abi<float>(const Geom&, double, const void*, const void*, void*, int, const double*, bool,
+                                       cudaStream_t, int);
+template void launch_wilson_abi<H16>(const Geom&, double, const void*, const void*, void*, int, const double*, bool,
+                                     cudaStream_t, int);
+template void launch_wilson_abi<B16>(const Geom&, double, const void*, const void*, void*, int, const double*, bool,
+                                     cudaStream_t, int);
+
+template <typename S>
+void launch_dslash(const Geom& g, double m0, const void* links, const void* in, void* out, int nrhs,
+                   const double* d_phase, const Epilogue& e, cudaStream_t s, bool deriv, int shape) {
+    using R = typename Arith<S>::type;
+    const Args<R> a = make_args<S>(g, m0, links, in, out, d_phase, e);
     const bool dense = (shape & kShapeDense) != 0;
     int by = (shape & kShapeRhsMask) > 0 ? (shape & kShapeRhsMask) : (nrhs > 1 ? 2 : 1);
     while (by > 1 && by > nrhs) by >>= 1;

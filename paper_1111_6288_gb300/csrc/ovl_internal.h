@@ -84,6 +84,13 @@ void launch_dslash(const Geom& g, double m0, const void* links, const void* in, 
                    const double* d_phase, const Epilogue& e, cudaStream_t s, bool deriv = false,
                    int shape = 0);
 
+// One application of H_w (g5: D_w = gamma5 H_w) for the caller: out in the ABI layout [rhs][site][12]
+// (complex128 for S = double, else complex64); in: FP64 the same layout, else the internal planes of S.  The
+// result of a 16-bit S is rounded to its format.
+template <typename S>
+void launch_wilson_abi(const Geom& g, double m0, const void* links, const void* in, void* out, int nrhs,
+                       const double* d_phase, bool g5, cudaStream_t s, int shape = 0);
+
 // ---- kernels: fx.cu ---------------------------------------------------------
 // FP64 recurrences on site-scaled fixed-point vectors (fx_arith.h).  A vector of one right-hand side
 // takes fx_rhs_bytes(V) bytes; the links (from the FP64 links, boundary signs folded in) fx_link_bytes(V),
@@ -117,7 +124,8 @@ void launch_fx_dslash(const Geom& g, const FxLinks& U, const void* in, void* out
                       const FxEpilogue& e, cudaStream_t s, int shape = 0);
 
 // ---- kernels: blas.cu -----------------------------------------------------
-// ABI spinor [rhs][site][12] (dtype_in: 0 complex128, 1 complex64) -> internal [rhs][12][V] of R.
+// ABI spinor [rhs][site][12] (dtype_in: 0 complex128, 1 complex64) -> internal [rhs][12][V] of R (double,
+// float, or rounded to H16 / B16 storage).
 template <typename R>
 void launch_pack_spinor(const void* abi, int dtype_in, void* internal, int V, int nrhs, cudaStream_t s);
 template <typename R>
