@@ -302,10 +302,10 @@ int ov_set_eigensolver_memory(ov_ctx* ctx, long long bytes);
 int ov_project_small(ov_ctx* ctx, double phase, const void* in, void* ys, void* xperp, int nrhs,
                      ov_stream_t stream);
 
-/* How FP32 projections of 8 or more vectors run: 0 = on the faster of the two paths, timed once per
- * (bank size, batch size) on the call's own buffers (ov_tune_info lists the times); 1 = CUDA cores;
- * 2 = tensor cores (tcgen05, TF32 with a three-term split for FP32 accuracy; bank size <= 384).
- * FP64 projections and batches below 8 always use the CUDA cores.  Default 0. */
+/* How FP32 projections of 8 or more vectors run: 1 = CUDA cores; 0 and 2 = tensor cores (tcgen05, TF32
+ * with a three-term split for FP32 accuracy; bank size <= 384), 0 falling back to the CUDA cores where
+ * the tensor-core path is not available.  FP64 projections and batches below 8 always use the CUDA
+ * cores.  ov_tune_info lists the sizes that took the tensor cores.  Default 0. */
 int ov_set_projection(ov_ctx* ctx, int method);
 
 /* ---- propagator solve (Sec. 3.2) --------------------------------------- */

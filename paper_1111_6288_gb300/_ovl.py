@@ -284,7 +284,7 @@ class Context:
         self.params.inner_precision = int(precision)
 
     def set_projection(self, method):
-        """FP32 small-space projections of 8+ vectors: 0 timed choice, 1 CUDA cores, 2 tensor cores."""
+        """FP32 small-space projections of 8+ vectors: 1 CUDA cores, 0 (where available) and 2 tensor cores."""
         _check(lib().ov_set_projection(self.handle, int(method)), self.handle)
 
     def set_eigensolver_memory(self, nbytes):

@@ -23,6 +23,7 @@
 #include <cstring>
 #include <map>
 #include <numeric>
+#include <set>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -126,10 +127,10 @@ struct ov_ctx {
     bool use_graphs = true;
     // autotuned right-hand sides per Wilson-kernel block, keyed by precision and systems
     std::map<std::pair<int, int>, int> launch_shape;
-    // small-space projection of FP32 vectors: 0 = timed per (bank size, batch), 1 = CUDA cores,
-    // 2 = tensor cores; the timed choice per (bank size, batch)
+    // small-space projection of 8 or more FP32 vectors: 1 = CUDA cores, 0 and 2 = tensor cores; the
+    // (bank size, batch) pairs in the tuning log
     int proj_method = 0;
-    std::map<std::pair<int, int>, int> proj_choice;
+    std::set<std::pair<int, int>> proj_seen;
     // working-set budget of the eigensolver's chunked passes (filter recurrence, residuals)
     long long eig_chunk_bytes = 16000000000LL;
     Buf tc_img;  // pre-split coefficients of the tensor-core projection
@@ -534,8 +535,9 @@ constexpr int kTcMinBatch = 8;
 
 // The small-space projection of k vectors (precision R, internal layout) on the bank b:
 // C = V^+ X, Xp = X - V C, Ys = V diag(s) C.  FP32 batches of kTcMinBatch or more vectors go through
-// the tcgen05 kernels when the context's method says so, or, by default, when they measured faster for
-// this (bank size, batch) the first time it appeared (both paths timed on the call's own buffers).
+// the tcgen05 kernels unless the context's method says otherwise: these were 2 to 20 times faster wherever
+// both were timed (batches of 8 and 24; 16 to 131072 sites, banks of 1 to 200: 31 against 93 us at the small
+// end, 0.67 against 1.5 ms for 3 vectors' bank and 8 vectors at 16^3 x 32).
 template <typename R>
 int project_bank(ov_ctx* c, const Bank* b, const void* X, int k, void* Xp, void* Ys, cudaStream_t s) {
     const int N = b->n;
@@ -543,10 +545,8 @@ int project_bank(ov_ctx* c, const Bank* b, const void* X, int k, void* Xp, void*
     const void* Vb = std::is_same<R, double>::value ? b->V64 : b->V32;
     TRY(ensure_small(c, 2LL * N * k, std::max<long long>((long long)N * 4 * 4 * 152, 152LL * N * std::min(k, 32)),
                      std::max(k, 1)));
-    int method = 1;
-    if (std::is_same<R, float>::value && k >= kTcMinBatch && N <= kTcMaxBank && tc_project_available())
-        method = c->proj_method;
-    if (method == 1) {
+    if (!std::is_same<R, float>::value || k < kTcMinBatch || N > kTcMaxBank || c->proj_method == 1 ||
+        !tc_project_available()) {
         small_space_project<R>(Vb, N, b->d_signs, X, k, Xp, Ys, n12, c->d_C, c->d_partial, c->partial_cap, s);
         CKL();
         return OV_OK;
@@ -562,41 +562,12 @@ int project_bank(ov_ctx* c, const Bank* b, const void* X, int k, void* Xp, void*
         CK(cudaMalloc(&c->tc_img.ptr, img));
         c->tc_img.bytes = img;
     }
-    auto run = [&](int m) -> cudaError_t {
-        if (m == 2)
-            return small_space_project_tc(Vb, N, b->d_signs, X, k, Xp, Ys, n12, c->d_C, c->d_partial, c->partial_cap,
-                                          c->tc_img.ptr, s);
-        small_space_project<R>(Vb, N, b->d_signs, X, k, Xp, Ys, n12, c->d_C, c->d_partial, c->partial_cap, s);
-        return cudaGetLastError();
-    };
-    if (method == 0) {
-        const auto key = std::make_pair(N, k);
-        auto it = c->proj_choice.find(key);
-        if (it == c->proj_choice.end()) {
-            cudaEvent_t e0, e1;
-            CK(cudaEventCreate(&e0));
-            CK(cudaEventCreate(&e1));
-            float ms[3] = {0.f, 0.f, 0.f};
-            for (int m : {1, 2}) {
-                CK(run(m));  // warm
-                CK(cudaEventRecord(e0, s));
-                for (int r = 0; r < 3; ++r) CK(run(m));
-                CK(cudaEventRecord(e1, s));
-                CK(cudaEventSynchronize(e1));
-                CK(cudaEventElapsedTime(&ms[m], e0, e1));
-            }
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            const int best = ms[2] < ms[1] ? 2 : 1;
-            char buf[128];
-            snprintf(buf, sizeof(buf), "projection N %d k %d: cuda cores %.1fus tensor cores %.1fus; ", N, k,
-                     1e3f * ms[1] / 3, 1e3f * ms[2] / 3);
-            c->tune_log += buf;
-            it = c->proj_choice.emplace(key, best).first;
-        }
-        method = it->second;
+    if (c->proj_seen.insert(std::make_pair(N, k)).second) {
+        char buf[96];
+        snprintf(buf, sizeof(buf), "projection N %d k %d: tensor cores; ", N, k);
+        c->tune_log += buf;
     }
-    CK(run(method));
+    CK(small_space_project_tc(Vb, N, b->d_signs, X, k, Xp, Ys, n12, c->d_C, c->d_partial, c->partial_cap, c->tc_img.ptr, s));
     return OV_OK;
 }
 

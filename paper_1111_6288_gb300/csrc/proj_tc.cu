@@ -165,29 +165,45 @@ __device__ __forceinline__ bool role_wait(uint32_t bar, uint32_t parity, volatil
     return true;
 }
 
-// 8 consecutive FP32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
-    uint32_t r[8];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// 8 consecutive FP32 columns of this thread's TMEM lane from each of four places, waited for once.
+__device__ __forceinline__ void tmem_ld8x4(uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3, float (&a)[8], float (&b)[8],
+                                           float (&c)[8], float (&d)[8]) {
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%32];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%33];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16, %17, %18, %19, %20, %21, %22, %23}, [%34];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24, %25, %26, %27, %28, %29, %30, %31}, [%35];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(t0), "r"(t1), "r"(t2), "r"(t3)
+        : "memory");
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 8; ++i) {
+        a[i] = __uint_as_float(r[i]);
+        b[i] = __uint_as_float(r[8 + i]);
+        c[i] = __uint_as_float(r[16 + i]);
+        d[i] = __uint_as_float(r[24 + i]);
+    }
 }
 
 // ---- C = V^+ X: split over the contraction ------------------------------------------------
 //
-// Grid (nchunk, ceil(na / 128)), 192 threads in three roles that hand tiles over through mbarriers:
+// Grid (nchunk, ceil(na / 128)), 448 threads in four roles that hand tiles over through mbarriers:
 //   warp 0   TMA producer: K-tile i of this block (32 floats of every row) into raw stage i % S,
 //            V rows [128 my, 128 my + 128) (rows beyond na arrive as zeros) and the KP rows of X;
 //   warp 1   MMA issuer (and TMEM owner): D = V [X; J X]^T, M = 128, N = 2 KP, three TF32 products
 //            per K-step, into the accumulator set of the tile's group of G K-tiles;
 //   warps 2-9  split each raw tile into the hi/lo operand tiles (the 128-byte swizzle keeps every
-//            16-byte chunk at its offset, J X too, rows KP..2KP-1), and add each completed group's
-//            accumulators into FP32 registers; at the end they write partial[cx][i][j] = (Re, Im).
+//            16-byte chunk at its offset, J X too, rows KP..2KP-1);
+//   warps 10-13  add each completed group's accumulators into FP32 registers; at the end they write
+//            partial[cx][i][j] = (Re, Im).
 // Barriers: full[s] (TMA bytes), empty[s] (the eight transform warps), opfull[b] (transform warps),
-// opempty[b] (MMA commit), accempty[set] (transform warps, once a group's sums are read).
+// opempty[b] (MMA commit), accfull[set] (MMA commit of a group's last tile), accempty[set] (the four
+// promotion warps, once a group's sums are read).
 template <int KP>
 struct VdotLayout {
     static constexpr int S = 6;
@@ -201,11 +217,15 @@ struct VdotLayout {
 };
 
 // Warp 0 TMA, warp 1 MMA and TMEM, warps 2-9 transform (two warps per scheduler hide each other's
-// shared-memory and conversion latency); warps w and w + 4 share TMEM lanes 32 (w % 4) .. and split the
-// accumulator columns.
-constexpr int WS_THREADS = 320;
+// shared-memory and conversion latency), warps 10-13 read the accumulators (warp w has TMEM lanes
+// 32 (w % 4) ..).  With the transform warps reading them too, the transform stood still meanwhile: 24
+// vectors on 100 modes of 16^3 x 32 took 1.69 ms for both kernels then and 0.92 ms now (1.05 ms before a_hi met
+// b_hi and b_lo in one MMA, which halves the reads of a_hi); DRAM 3-4 TB/s, bound by shared memory (raw tile
+// in, operand tiles out, MMA reads: about 1100 of 1300 clocks a K-tile) and the conversions (490 clocks).
+constexpr int WS_THREADS = 448;
 constexpr int NXW = 8;                 // transform warps
 constexpr int NXT = NXW * 32;          // transform threads
+constexpr int NAW = 4;                 // accumulator warps
 
 template <int KP>
 __global__ void __launch_bounds__(WS_THREADS, 1)
@@ -218,8 +238,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* raw = base;
     unsigned char* op = base + S * L::RAW;
-    uint64_t* bars = (uint64_t*)(op + 2 * L::OP);  // full[S], empty[S], opfull[2], opempty[2], accempty[2]
-    int* flags = (int*)(bars + 2 * S + 6);        // abort, issued, consumed, committed
+    uint64_t* bars = (uint64_t*)(op + 2 * L::OP);  // full[S], empty[S], opfull[2], opempty[2], accempty[2], accfull[2]
+    int* flags = (int*)(bars + 2 * S + 8);        // abort, issued, consumed, committed
     uint32_t* tslot = (uint32_t*)(flags + 4);
     volatile int* abort_flag = flags;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -234,7 +254,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
         return;
     }
     const uint32_t full0 = su32(bars), empty0 = full0 + 8 * S, opfull0 = empty0 + 8 * S, opempty0 = opfull0 + 16,
-                   accempty0 = opempty0 + 16;
+                   accempty0 = opempty0 + 16, accfull0 = accempty0 + 16;
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
             bar_init(full0 + 8 * s, 1);
@@ -243,7 +263,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
         for (int b = 0; b < 2; ++b) {
             bar_init(opfull0 + 8 * b, NXW);
             bar_init(opempty0 + 8 * b, 1);
-            bar_init(accempty0 + 8 * b, NXW);
+            bar_init(accempty0 + 8 * b, NAW);
+            bar_init(accfull0 + 8 * b, 1);
         }
         flags[0] = 0;
         flags[1] = flags[2] = flags[3] = 0;
@@ -256,7 +277,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
-    constexpr uint32_t IDESC = tf32_idesc(128, 2 * KP);
+    constexpr uint32_t IDESC = tf32_idesc(128, 2 * KP), IDESC2 = tf32_idesc(128, 4 * KP);
     if (warp == 0) {
         if (lane == 0) {  // producer
             int i = 0;
@@ -279,66 +300,64 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                 if (i % G == 0 && g >= 2 && !role_wait(accempty0 + 8 * set, ((g - 2) >> 1) & 1, abort_flag)) break;
                 tc_fence_after();
                 unsigned char* ob = op + b * L::OP;
-                const uint32_t a_hi = su32(ob), a_lo = a_hi + L::OPA, b_hi = a_hi + 2 * L::OPA, b_lo = b_hi + L::OPB;
+                // a_hi against the rows of b_hi and, behind them, b_lo, into both accumulators at once
+                const uint32_t a_hi = su32(ob), a_lo = a_hi + L::OPA, b_hi = a_hi + 2 * L::OPA;
                 const uint32_t big = tmem + set * 4 * KP, small = big + 2 * KP;
 #pragma unroll
                 for (int ks = 0; ks < KT / 8; ++ks) {
                     const uint32_t o = ks * 32;  // 8 TF32 of K: 32 bytes along the swizzled row
                     const uint32_t more = (i % G > 0 || ks > 0) ? 1u : 0u;
-                    mma_tf32(big, sw128_desc(a_hi + o), sw128_desc(b_hi + o), IDESC, more);
-                    mma_tf32(small, sw128_desc(a_hi + o), sw128_desc(b_lo + o), IDESC, more);
+                    mma_tf32(big, sw128_desc(a_hi + o), sw128_desc(b_hi + o), IDESC2, more);
                     mma_tf32(small, sw128_desc(a_lo + o), sw128_desc(b_hi + o), IDESC, 1u);
                 }
                 mma_commit(opempty0 + 8 * b);
+                if (i % G == G - 1 || i == nt - 1) mma_commit(accfull0 + 8 * set);
             }
             flags[3] = i;
         }
-    } else {  // warps 2-9: transform and promotion
-        const int t = tid - 64;
-        // Warp w reads TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31; of the two warps on a quarter, the first
-        // keeps the real parts (columns j), the second the imaginary parts (KP + j).
-        const int half = (warp - 2) >> 2;
-        const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        float acc[KP];
-#pragma unroll
-        for (int q = 0; q < KP; ++q) acc[q] = 0.f;
+    } else if (warp >= 2 + NXW) {  // warps 10-13: promotion
         // The tensor core rounds its accumulation steps toward zero, a bias that grows with the steps
         // summed in one accumulator: each group of G K-tiles has fresh accumulators, added here into
         // FP32 registers with round-to-nearest.
-        auto promote = [&](int set) {
+        const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        float re[KP], im[KP];
+#pragma unroll
+        for (int q = 0; q < KP; ++q) re[q] = im[q] = 0.f;
+        const int ngroups = (nt + G - 1) / G;
+        int g = 0;
+        for (; g < ngroups; ++g) {
+            const int set = g & 1;
+            if (!__all_sync(0xffffffffu, role_wait(accfull0 + 8 * set, (g >> 1) & 1, abort_flag))) break;
+            tc_fence_after();
+            const uint32_t big = tlane + set * 4 * KP, small = big + 2 * KP;
 #pragma unroll
             for (int c0 = 0; c0 < KP; c0 += 8) {
-                float v[8], w[8];
-                tmem_ld8(tlane + set * 4 * KP + half * KP + c0, v);
-                tmem_ld8(tlane + set * 4 * KP + 2 * KP + half * KP + c0, w);
+                float v[8], w[8], vi[8], wi[8];
+                tmem_ld8x4(big + c0, small + c0, big + KP + c0, small + KP + c0, v, w, vi, wi);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) acc[c0 + q] += v[q] + w[q];
+                for (int q = 0; q < 8; ++q) {
+                    re[c0 + q] += v[q] + w[q];
+                    im[c0 + q] += vi[q] + wi[q];
+                }
             }
-        };
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) bar_arrive(accempty0 + 8 * set);
+        }
+        const int m = row0 + (warp & 3) * 32 + lane;
+        if (g == ngroups && m < na) {
+#pragma unroll
+            for (int j = 0; j < KP; ++j)
+                if (j < nb) partial[((long long)cx * na + m) * nb + j] = make_double2((double)re[j], (double)im[j]);
+        }
+    } else {  // warps 2-9: transform
+        const int t = tid - 64;
         constexpr int XC = KP * ROW_BYTES / 16;  // 16-byte chunks of the X tile
-        int promoted = 0, i = 0;
-        bool ok = true;
+        int i = 0;
         for (; i < nt; ++i) {
             const int s = i % S, b = i & 1;
-            if (!role_wait(full0 + 8 * s, (i / S) & 1, abort_flag)) {
-                ok = false;
-                break;
-            }
-            if (i >= 2) {
-                if (!role_wait(opempty0 + 8 * b, ((i - 2) >> 1) & 1, abort_flag)) {
-                    ok = false;
-                    break;
-                }
-                if ((i - 2) % G == G - 1) {  // tile i - 2 completed its group
-                    const int set = ((i - 2) / G) & 1;
-                    tc_fence_after();
-                    promote(set);
-                    ++promoted;
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) bar_arrive(accempty0 + 8 * set);
-                }
-            }
+            if (!role_wait(full0 + 8 * s, (i / S) & 1, abort_flag)) break;
+            if (i >= 2 && !role_wait(opempty0 + 8 * b, ((i - 2) >> 1) & 1, abort_flag)) break;
             const float4* rv = (const float4*)(raw + s * L::RAW);
             const float4* rx = (const float4*)(raw + s * L::RAW + L::RAW_V);
             unsigned char* ob = op + b * L::OP;
@@ -371,18 +390,6 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             }
         }
         if (t == 0) flags[2] = i;
-        if (ok && role_wait(opempty0 + 8 * ((nt - 1) & 1), ((nt - 1) >> 1) & 1, abort_flag)) {
-            tc_fence_after();
-            const int ngroups = (nt + G - 1) / G;  // at most the last two are not added yet
-            for (int gi = promoted; gi < ngroups; ++gi) promote(gi & 1);
-            const int m = row0 + (warp & 3) * 32 + lane;
-            double* pd = (double*)partial;
-            if (m < na) {
-#pragma unroll
-                for (int j = 0; j < KP; ++j)
-                    if (j < nb) pd[2 * (((long long)cx * na + m) * nb + j) + half] = (double)acc[j];
-            }
-        }
     }
     __syncthreads();
     if (*abort_flag && tid == 0) {  // before the block exits: copies and MMAs it started must be done
@@ -473,11 +480,10 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                const float2* __restrict__ X, float2* __restrict__ Xp, float2* __restrict__ Ys, long long n, int nb,
                int mtiles) {
     // Roles as in vdot_tc_k: warp 0 TMA (the raw V tile and, by a 1-D bulk copy, the K-tile's
-    // coefficient image), warp 1 MMA issue and TMEM, warps 2-9 the transposing split of V and the
-    // epilogue.  Steps u run over this block's output tiles (blockIdx.x, + gridDim.x, ...) and their
+    // coefficient image), warp 1 MMA issue and TMEM, warps 2-9 the transposing split of V, warps 10-13
+    // the epilogue, whose loads of X are on their way while it waits for the accumulator.  Steps u run over this block's output tiles (blockIdx.x, + gridDim.x, ...) and their
     // K-tiles; the MMAs read the coefficient image in the raw stage, so a stage is released by the MMA
-    // commit.  Output tiles alternate between two accumulator sets, each {hi x hi: 4 KP | small: 4 KP};
-    // the epilogue of tile q runs after the first K-tile of tile q + 1 has been handed to the MMAs.
+    // commit.  Output tiles alternate between two accumulator sets, each {hi x hi: 4 KP | small: 4 KP}.
     using L = ApplyLayout<KP>;
     static_assert(KP % 8 == 0 && KP >= 8 && KP <= 32, "KP");
     constexpr int S = L::S;
@@ -504,7 +510,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             bar_init(opfull0 + 8 * b, NXW);
             bar_init(opempty0 + 8 * b, 1);
             bar_init(accfull0 + 8 * b, 1);
-            bar_init(accempty0 + 8 * b, NXW);
+            bar_init(accempty0 + 8 * b, NAW);
         }
         flags[0] = 0;
         flags[1] = flags[2] = flags[3] = 0;
@@ -516,7 +522,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
-    constexpr uint32_t IDESC = tf32_idesc(128, 4 * KP);
+    constexpr uint32_t IDESC = tf32_idesc(128, 4 * KP), IDESC2 = tf32_idesc(128, 8 * KP);
     if (warp == 0) {
         if (lane == 0) {  // producer
             int u = 0;
@@ -539,14 +545,13 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
                 if (kt == 0 && q >= 2 && !role_wait(accempty0 + 8 * ts, ((q - 2) >> 1) & 1, abort_flag)) break;
                 tc_fence_after();
                 const uint32_t a_hi = su32(op + b * L::OP), a_lo = a_hi + L::OPA;
-                const uint32_t b_hi = su32(raw + s * L::RAW + L::RAW_V), b_lo = b_hi + L::BIMG / 2;
+                const uint32_t b_hi = su32(raw + s * L::RAW + L::RAW_V);  // b_lo's rows follow b_hi's
                 const uint32_t big = tmem + ts * 8 * KP, small = big + 4 * KP;
 #pragma unroll
                 for (int ks = 0; ks < KT / 8; ++ks) {
                     const uint32_t o = ks * 32;
                     const uint32_t more = (kt > 0 || ks > 0) ? 1u : 0u;
-                    mma_tf32(big, sw128_desc(a_hi + o), sw128_desc(b_hi + o), IDESC, more);
-                    mma_tf32(small, sw128_desc(a_hi + o), sw128_desc(b_lo + o), IDESC, more);
+                    mma_tf32(big, sw128_desc(a_hi + o), sw128_desc(b_hi + o), IDESC2, more);
                     mma_tf32(small, sw128_desc(a_lo + o), sw128_desc(b_hi + o), IDESC, 1u);
                 }
                 mma_commit(opempty0 + 8 * b);  // the operand buffer is free
@@ -555,58 +560,47 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             }
             flags[3] = u;
         }
-    } else {  // warps 2-9: transposing split and epilogue
-        const int t = tid - 64;
+    } else if (warp >= 2 + NXW) {  // warps 10-13: epilogue
         const int q4 = warp & 3;  // TMEM lanes 32 q4 .. 32 q4 + 31
         const uint32_t tlane = tmem + ((uint32_t)(q4 * 32) << 16);
-        auto epilogue = [&](int q) -> bool {  // output tile q of this block
-            const int ts = q & 1;
-            if (!role_wait(accfull0 + 8 * ts, (q >> 1) & 1, abort_flag)) return false;
-            tc_fence_after();
-            const int mt = (int)blockIdx.x + q * (int)gridDim.x;
+        for (int q = 0; q < nmt; ++q) {
+            const int ts = q & 1, mt = (int)blockIdx.x + q * (int)gridDim.x;
             const long long pos = (long long)mt * 128 + q4 * 32 + lane;
-            const uint32_t tl = tlane + ts * 8 * KP;
-#pragma unroll 1
-            for (int j0 = 8 * ((warp - 2) >> 2); j0 < KP; j0 += 16) {  // the quarter's two warps alternate
-                float r1[8], i1[8], r2[8], i2[8], w[8];
-                tmem_ld8(tl + j0, r1);
-                tmem_ld8(tl + KP + j0, i1);
-                tmem_ld8(tl + 2 * KP + j0, r2);
-                tmem_ld8(tl + 3 * KP + j0, i2);
-                tmem_ld8(tl + 4 * KP + j0, w);
+            float2 x[KP];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) r1[e] += w[e];
-                tmem_ld8(tl + 5 * KP + j0, w);
+            for (int j = 0; j < KP; ++j) x[j] = pos < n && j < nb ? X[(long long)j * n + pos] : make_float2(0.f, 0.f);
+            if (!__all_sync(0xffffffffu, role_wait(accfull0 + 8 * ts, (q >> 1) & 1, abort_flag))) break;
+            tc_fence_after();
+            const uint32_t big = tlane + ts * 8 * KP, small = big + 4 * KP;
 #pragma unroll
-                for (int e = 0; e < 8; ++e) i1[e] += w[e];
-                tmem_ld8(tl + 6 * KP + j0, w);
+            for (int j0 = 0; j0 < KP; j0 += 8) {
+                float r1[8], i1[8], w1[8], w2[8];
+                tmem_ld8x4(big + j0, small + j0, big + KP + j0, small + KP + j0, r1, w1, i1, w2);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) r2[e] += w[e];
-                tmem_ld8(tl + 7 * KP + j0, w);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) i2[e] += w[e];
+                for (int e = 0; e < 8; ++e) {
+                    x[j0 + e].x += r1[e] + w1[e];
+                    x[j0 + e].y += i1[e] + w2[e];
+                }
+                tmem_ld8x4(big + 2 * KP + j0, small + 2 * KP + j0, big + 3 * KP + j0, small + 3 * KP + j0, r1, w1, i1, w2);
                 if (pos < n) {
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int j = j0 + e;
-                        if (j < nb) {
-                            const long long o = (long long)j * n + pos;
-                            const float2 x = X[o];
-                            Xp[o] = make_float2(x.x + r1[e], x.y + i1[e]);
-                            Ys[o] = make_float2(r2[e], i2[e]);
+                    for (int e = 0; e < 8; ++e)
+                        if (j0 + e < nb) {
+                            const long long o = (long long)(j0 + e) * n + pos;
+                            Xp[o] = x[j0 + e];
+                            Ys[o] = make_float2(r1[e] + w1[e], i1[e] + w2[e]);
                         }
-                    }
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) bar_arrive(accempty0 + 8 * ts);
-            return true;
-        };
+        }
+    } else {  // warps 2-9: transposing split
+        const int t = tid - 64;
         int u = 0;
-        bool ok = true;
-        for (; u < nsteps && ok; ++u) {
-            const int s = u % S, b = u & 1, kt = u % nkt, q = u / nkt;
+        for (; u < nsteps; ++u) {
+            const int s = u % S, b = u & 1;
             if (!role_wait(full0 + 8 * s, (u / S) & 1, abort_flag)) break;
             if (u >= 2 && !role_wait(opempty0 + 8 * b, ((u - 2) >> 1) & 1, abort_flag)) break;
             // thread t builds half a row of A
@@ -626,10 +620,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1)
             fence_async_smem();
             __syncwarp();
             if (lane == 0) bar_arrive(opfull0 + 8 * b);
-            if (kt == 0 && q >= 1) ok = epilogue(q - 1);
         }
         if (t == 0) flags[2] = u;
-        if (ok && u == nsteps) epilogue(nmt - 1);
     }
     __syncthreads();
     if (*abort_flag && tid == 0) {  // before the block exits: copies and MMAs it started must be done
