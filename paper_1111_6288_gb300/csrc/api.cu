@@ -1303,7 +1303,7 @@ int ov_set_gauge(ov_ctx* c, const void* U, int dtype, ov_stream_t stream) {
     if (!c->U64) {
         if (cudaMalloc(&c->U64, n * sizeof(double2)) != cudaSuccess ||
             cudaMalloc(&c->U32, 4ull * 3 * c->g.V * sizeof(float4)) != cudaSuccess ||
-            (half && cudaMalloc(&c->U16, 96ull * c->g.V) != cudaSuccess)) {
+            (half && cudaMalloc(&c->U16, 144ull * c->g.V) != cudaSuccess)) {
             cudaGetLastError();
             return fail(c, OV_ERR_OOM, "gauge field allocation failed");
         }

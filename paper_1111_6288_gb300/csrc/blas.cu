@@ -225,9 +225,9 @@ __global__ void pack_gauge_half_k(const TI* __restrict__ abi, void* __restrict__
     if (idx >= 4LL * V) return;
     const int mu = (int)(idx / V), s = (int)(idx % V);
     const TI* src = abi + ((long long)mu * V + s) * 9;
-    float2 r[6];
+    float2 r[9];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) r[k] = make_float2((float)src[k].x, (float)src[k].y);
+    for (int k = 0; k < 9; ++k) r[k] = make_float2((float)src[k].x, (float)src[k].y);
     half_store_link<S>(out, V, mu, s, r);
 }
 

@@ -7,7 +7,7 @@
 //   FP64 links   [4][9][V]    double2, entry 3*a + b of U_mu(n)
 //   FP32 links   [4][3][V]    float4 = rows 0 and 1 of U_mu(n); row 2 = conj(row0 x row1)
 //   FP16 / BF16  spinors [rhs][3][V] uint4 (+ a float scale per site for FP16) and links
-//                rows 0 and 1 in 24 bytes, FP32 arithmetic (half_store.h)
+//                in 36 bytes, FP32 arithmetic (half_store.h)
 //   bank         [n_ev][...]  the spinor layout of its precision
 // A spinor vector is 12 V complex numbers (192 B or 96 B per site) in both precisions,
 // so element-wise kernels and inner products treat vectors as flat complex arrays.
