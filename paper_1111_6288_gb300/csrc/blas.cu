@@ -235,6 +235,21 @@ __global__ void pack_gauge_half_k(const TI* __restrict__ abi, void* __restrict__
 
 constexpr int RT = 256;
 
+// (re, im) += a b, and conj(a) b, four fused multiply-adds (written as sums of products they are six
+// operations: nvcc fuses within a product's sum only)
+__device__ __forceinline__ float fmad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fmad(double a, double b, double c) { return __fma_rn(a, b, c); }
+template <typename R, typename T>
+__device__ __forceinline__ void mac(R& re, R& im, T a, T b) {
+    re = fmad(-a.y, b.y, fmad(a.x, b.x, re));
+    im = fmad(a.y, b.x, fmad(a.x, b.y, im));
+}
+template <typename R, typename T>
+__device__ __forceinline__ void mac_conj(R& re, R& im, T a, T b) {
+    re = fmad(a.y, b.y, fmad(a.x, b.x, re));
+    im = fmad(-a.y, b.x, fmad(a.x, b.y, im));
+}
+
 // partial[r][b] = sum over this block's slice of conj(a) b (rhs r)
 template <typename R, bool NORM>
 __global__ void __launch_bounds__(RT) dot_partial_k(const typename C2<R>::T* __restrict__ a,
@@ -247,11 +262,10 @@ __global__ void __launch_bounds__(RT) dot_partial_k(const typename C2<R>::T* __r
     for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < n; i += (long long)gridDim.x * RT) {
         typename C2<R>::T x = pa[i];
         if (NORM) {
-            sre += x.x * x.x + x.y * x.y;
+            sre = fmad(x.y, x.y, fmad(x.x, x.x, sre));
         } else {
             typename C2<R>::T y = pb[i];
-            sre += x.x * y.x + x.y * y.y;
-            sim += x.x * y.y - x.y * y.x;
+            mac_conj(sre, sim, x, y);
         }
     }
     double2 tot = block_sum<RT>(make_double2((double)sre, (double)sim));
@@ -364,14 +378,26 @@ constexpr int MT = 8;      // vectors per tile, both sides
 constexpr int MK = 32;     // elements per slab
 constexpr int MNT = 256;   // threads
 
-template <typename R>
+// HERM: A and B are the same vectors; only tiles on and above the diagonal are computed (blockIdx.y counts
+// them row by row), and each writes its mirror image as well.  In FP64 the FP64 pipe is the bound: the Gram
+// matrix of 32 vectors of 8^3 x 16 took 944 us with all tiles and six operations a product, 867 with the upper
+// tiles, and takes 431 us with four fused operations and as many blocks as fill the SMs evenly.
+template <typename R, bool HERM>
 __global__ void __launch_bounds__(MNT) multidot_k(const typename C2<R>::T* __restrict__ A, long long sA, int na,
                                                   const typename C2<R>::T* __restrict__ B, long long sB, int nb,
                                                   long long n, long long chunk, double2* __restrict__ partial) {
     __shared__ typename C2<R>::T shA[MT][MK + 1];
     __shared__ typename C2<R>::T shB[MT][MK + 1];
     __shared__ double2 red[MNT];
-    const int i0 = blockIdx.y * MT, j0 = blockIdx.z * MT;
+    int ti = blockIdx.y, tj = blockIdx.z;
+    if constexpr (HERM) {
+        const int nt = (na + MT - 1) / MT;
+        tj = ti;
+        ti = 0;
+        while (tj >= nt - ti) tj -= nt - ti++;
+        tj += ti;
+    }
+    const int i0 = ti * MT, j0 = tj * MT;
     const long long k_begin = (long long)blockIdx.x * chunk;
     const long long k_end = min(n, k_begin + chunk);
     const int t = threadIdx.x;
@@ -394,9 +420,7 @@ __global__ void __launch_bounds__(MNT) multidot_k(const typename C2<R>::T* __res
         __syncthreads();
 #pragma unroll
         for (int e = part * 8; e < part * 8 + 8; ++e) {
-            typename C2<R>::T a = shA[pi][e], b = shB[pj][e];
-            sre += a.x * b.x + a.y * b.y;
-            sim += a.x * b.y - a.y * b.x;
+            mac_conj(sre, sim, shA[pi][e], shB[pj][e]);
         }
         __syncthreads();
     }
@@ -408,7 +432,10 @@ __global__ void __launch_bounds__(MNT) multidot_k(const typename C2<R>::T* __res
         v = dadd(v, red[t + 128]);
         v = dadd(v, red[t + 192]);
         const int i = i0 + (t >> 3), j = j0 + (t & 7);
-        if (i < na && j < nb) partial[((long long)blockIdx.x * na + i) * nb + j] = v;
+        if (i < na && j < nb) {
+            partial[((long long)blockIdx.x * na + i) * nb + j] = v;
+            if (HERM && ti != tj) partial[((long long)blockIdx.x * na + j) * nb + i] = make_double2(v.x, -v.y);
+        }
     }
 }
 
@@ -416,6 +443,7 @@ __global__ void multidot_sum_k(const double2* __restrict__ partial, int nchunk, 
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= nab) return;
     double2 v = make_double2(0, 0);
+#pragma unroll 8
     for (int c = 0; c < nchunk; ++c) v = dadd(v, partial[(long long)c * nab + idx]);
     C[idx] = v;
 }
@@ -442,13 +470,12 @@ __global__ void __launch_bounds__(256) combine_k(const typename C2<R>::T* __rest
         R accr[CJT], acci[CJT];
 #pragma unroll
         for (int j = 0; j < CJT; ++j) accr[j] = acci[j] = 0;
+#pragma unroll 4
         for (int i = 0; i < na; ++i) {
             typename C2<R>::T a = A[(long long)i * sA + m];
 #pragma unroll
             for (int j = 0; j < CJT; ++j) {
-                const typename C2<R>::T c = shC[i * CJT + j];
-                accr[j] += a.x * c.x - a.y * c.y;
-                acci[j] += a.x * c.y + a.y * c.x;
+                mac(accr[j], acci[j], a, shC[i * CJT + j]);
             }
         }
         for (int j = 0; j < nj; ++j) {
@@ -501,8 +528,7 @@ __global__ void __launch_bounds__(256) vdot_rows_k(const typename C2<R>::T* __re
                 const typename C2<R>::T v = V[(long long)i * sV + m];
 #pragma unroll
                 for (int j = 0; j < NB; ++j) {  // conj(v) * x
-                    ar[r][j] += v.x * xv[j].x + v.y * xv[j].y;
-                    ai[r][j] += v.x * xv[j].y - v.y * xv[j].x;
+                    mac_conj(ar[r][j], ai[r][j], v, xv[j]);
                 }
             }
         }
@@ -550,10 +576,8 @@ __global__ void __launch_bounds__(256) proj_apply_k(const typename C2<R>::T* __r
 #pragma unroll
             for (int j = 0; j < NB; ++j) {
                 const typename C2<R>::T c1 = cn[i * NB + j], c2 = cs[i * NB + j];
-                a1r[j] += v.x * c1.x - v.y * c1.y;
-                a1i[j] += v.x * c1.y + v.y * c1.x;
-                a2r[j] += v.x * c2.x - v.y * c2.y;
-                a2i[j] += v.x * c2.y + v.y * c2.x;
+                mac(a1r[j], a1i[j], v, c1);
+                mac(a2r[j], a2i[j], v, c2);
             }
         }
 #pragma unroll
@@ -750,19 +774,25 @@ void multidot(const void* A, long long strideA, int na, const void* B, long long
         return;
     }
     const int ti = (na + MT - 1) / MT, tj = (nb + MT - 1) / MT;
-    // enough chunks to fill the GPU about four times over, bounded by the partial buffer
-    // enough chunks to fill the GPU, and chunks of at most 4096 elements (each thread's partial
+    const bool herm = A == B && na == nb && strideA == strideB;
+    const int tiles = herm ? ti * (ti + 1) / 2 : ti * tj;
+    // chunks that fill the GPU about four times over (not a block more: one SM with five takes a quarter
+    // longer), bounded by the partial buffer, and chunks of at most 4096 elements (each thread's partial
     // sum then covers about 1000 products, short enough for FP32 accumulation)
-    long long nchunk = std::max((4LL * 152 + ti * tj - 1) / (ti * tj), (n + 4095) / 4096);
+    long long nchunk = std::max(4LL * 152 / tiles, (n + 4095) / 4096);
     const long long max_chunk_by_cap = partial_cap / ((long long)na * nb);
     if (nchunk > max_chunk_by_cap) nchunk = max_chunk_by_cap;
     if (nchunk < 1) nchunk = 1;
     long long chunk = (n + nchunk - 1) / nchunk;
     chunk = ((chunk + MK - 1) / MK) * MK;
     nchunk = (n + chunk - 1) / chunk;
-    dim3 grid((unsigned)nchunk, ti, tj);
-    multidot_k<R><<<grid, MNT, 0, s>>>((const typename C2<R>::T*)A, strideA, na, (const typename C2<R>::T*)B, strideB,
-                                       nb, n, chunk, d_partial);
+    typedef typename C2<R>::T T;
+    if (herm)
+        multidot_k<R, true><<<dim3((unsigned)nchunk, tiles), MNT, 0, s>>>((const T*)A, strideA, na, (const T*)B, strideB, nb,
+                                                                         n, chunk, d_partial);
+    else
+        multidot_k<R, false><<<dim3((unsigned)nchunk, ti, tj), MNT, 0, s>>>((const T*)A, strideA, na, (const T*)B, strideB,
+                                                                           nb, n, chunk, d_partial);
     count_launch();
     const int nab = na * nb;
     multidot_sum_k<<<(nab + 255) / 256, 256, 0, s>>>(d_partial, (int)nchunk, nab, d_C);
@@ -780,10 +810,14 @@ void combine(const void* A, long long strideA, int na, const double2* d_C, int l
         count_launch();
         return;
     }
+    // FP64: blocks of 64, so that the FP64 pipes of all SMs end together.  8 columns from 32 vectors of
+    // 8^3 x 16: 299 us with 384 blocks of 256 on the 152 SMs and six operations a product, 282 us with blocks of
+    // 64, 171 us with four operations as well, what the FP64 pipe takes for them.
+    constexpr int NT = std::is_same<R, double>::value ? 64 : 256;
     const size_t shm = sizeof(typename C2<R>::T) * (size_t)na * CJ;
     for (int j0 = 0; j0 < nb; j0 += CJ) {
         const int nj = (nb - j0 < CJ) ? nb - j0 : CJ;
-        combine_k<R, CJ><<<grid_for(n, 256, 152 * 8), 256, shm, s>>>(
+        combine_k<R, CJ><<<grid_for(n, NT, 152 * 8 * (256 / NT)), NT, shm, s>>>(
             (const typename C2<R>::T*)A, strideA, na, d_C, ldc, j0, nj, alpha, (const typename C2<R>::T*)X, strideX,
             (typename C2<R>::T*)out, strideO, n);
         count_launch();
