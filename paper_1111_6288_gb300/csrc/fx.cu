@@ -45,12 +45,12 @@ __device__ __forceinline__ void copy_wait() {
 // then its components of psi and of the three epilogue vectors.  Each warp copies the next step into
 // shared memory while it computes (the two lanes of a site share the copy of its link).
 //
-// Bound by the integer multiply pipe and the register reads behind it (per lane and site about 900
-// 32 x 32 + 64-bit multiply-adds of 2600 instructions; that pipe is 70 % busy), beyond L2 also by the
-// links (576 B a site, read 1.4 times).  Measured, mean of the two launches of a Clenshaw step against
-// dslash_kernel<double>: 51 against 231 us at 16^3 x 32, 39 against 180 us for 12 systems of 8^3 x 16,
-// 6.8 against 35 us on 4^4.  One thread a site instead of two lanes took 66 us at 16^3 x 32, operands
-// loaded straight into registers 65 us.
+// Bound by the integer pipes and the register reads behind them (per lane and site about 700 32 x 32 +
+// 64-bit multiply-adds of 2600 instructions), beyond L2 also by the links (576 B a site, read 1.4 times).
+// Measured, mean of the two launches of a Clenshaw step against dslash_kernel<double>: 48.5 against 231 us
+// at 16^3 x 32, 36.7 against 180 us for 12 systems of 8^3 x 16, 6.5 against 35 us on 4^4.  (With four limb
+// products a complex product and 51 us at 16^3 x 32, one thread a site instead of two lanes took 66 us and
+// operands loaded straight into registers 65 us.)
 template <bool EPI, bool DUAL>
 __global__ void __launch_bounds__(FX_THREADS, kBlocksPerSm) fx_dslash_kernel(const __grid_constant__ fx::Args a, int nrhs) {
     extern __shared__ int4 ring[];
