@@ -25,6 +25,11 @@ constexpr int FX_THREADS = 128;
 // four stages, two or five blocks are 5-15 % slower.
 constexpr int kStages = 2;
 constexpr int kBlocksPerSm = 4;
+// Launches of at most this many blocks of 16 sites go to fx_split_kernel: three on each of the 152 SMs, all it
+// has registers for.  Two lanes a site against eight: 6.6 / 5.1 us on 4^4 (16 blocks), 7.4 / 6.5 on 8^3 x 12,
+// 7.6 / 6.6 on 9^3 x 10 (456 blocks), 7.3 / 8.7 on 8^3 x 16 (512 blocks); the derivative 10.3 / 7.7 us on 4^3 x 8,
+// 11.4 / 9.3 on 9^3 x 10, 11.4 / 12.7 on 8^3 x 16.
+constexpr int kSplitBlocks = 3 * 152;
 constexpr int kSpinInt4 = 6 * 32;             // a lane's six components of a spinor
 constexpr int kStageInt4 = kSpinInt4 + 9 * 16;  // and the links of the warp's 16 sites
 constexpr int kWarpBytes = kStages * kStageInt4 * 16;
@@ -48,7 +53,7 @@ __device__ __forceinline__ void copy_wait() {
 // Bound by the integer pipes and the register reads behind them (per lane and site about 700 32 x 32 +
 // 64-bit multiply-adds of 2600 instructions), beyond L2 also by the links (576 B a site, read 1.4 times).
 // Measured, mean of the two launches of a Clenshaw step against dslash_kernel<double>: 48.5 against 231 us
-// at 16^3 x 32, 36.7 against 180 us for 12 systems of 8^3 x 16, 6.5 against 35 us on 4^4.  (With four limb
+// at 16^3 x 32, 36.7 against 180 us for 12 systems of 8^3 x 16, 6.6 against 35 us on 4^4.  (With four limb
 // products a complex product and 51 us at 16^3 x 32, one thread a site instead of two lanes took 66 us and
 // operands loaded straight into registers 65 us.)
 template <bool EPI, bool DUAL>
@@ -197,6 +202,127 @@ __global__ void __launch_bounds__(FX_THREADS, kBlocksPerSm) fx_dslash_kernel(con
         fx::store_spin(o, f, H.up);
         fx::store_spin(o, 2 + f, H.own);
         if (f == 0) *fx::exponent_at(a.out + off, s) = bad ? fx::kNanExp : E;
+    }
+}
+
+// The same on few sites, eight lanes a site: there a launch takes as long as one warp's instructions, one
+// every four to five cycles, whatever the memory does (a ring that holds every step took 6.1 us on 4^4 instead
+// of 6.4).  4^4: 6.6 -> 5.1 us.  A block has 16 sites; each of its four warps does the two hops of one direction, operands loaded
+// straight into registers, and the sums meet in shared memory, where each thread takes three of a site's 24
+// numbers through the epilogue.  The sums are integers, so the bits are those of fx_dslash_kernel.
+template <bool EPI, bool DUAL>
+__global__ void __launch_bounds__(128) fx_split_kernel(const __grid_constant__ fx::Args a) {
+    __shared__ i64 sums[4][24][17];
+    __shared__ int eref_of[16], e0_of[16];
+    const int V = a.V, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, f = lane >> 4;
+    const int first = blockIdx.x * 16, r = blockIdx.y;
+    const i64 off = (i64)r * fx::rhs_bytes(V);
+    const char* in = a.in + off;
+    // numbers 3 t .. 3 t + 2 of site first + j
+    const int j = threadIdx.x >> 3, t = threadIdx.x & 7, sj = min(first + j, V - 1);
+    auto number = [&](const char* v, int q) { return (const int2*)(fx::at(v, sj) + ((3 * t + q) >> 1) * fx::kTile) + ((3 * t + q) & 1); };
+    int2 x[3], x1[3], x2[3], x3[3];
+    int e1 = 0, e2 = 0, e3 = 0;
+    auto fetch = [&](const char* v, int2(&d)[3]) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) d[q] = v ? *number(v + off, q) : make_int2(0, 0);
+        return v ? *fx::exponent_at(v + off, sj) : 0;
+    };
+    fetch(a.in, x);
+    if constexpr (EPI) {
+        e1 = fetch(a.v1, x1);
+        e2 = fetch(a.v2, x2);
+        e3 = fetch(a.v3, x3);
+    }
+    fx::Half H;
+    const int s = min(first + (lane & 15), V - 1);
+    fx::half_setup(a, s, r, f, H);
+    if (threadIdx.x < 16) {
+        eref_of[threadIdx.x] = H.eref;
+        e0_of[threadIdx.x] = H.e0;
+    }
+    i64 fu[6], fl[6], bu[6], bl[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) fu[k] = fl[k] = bu[k] = bl[k] = 0;
+    auto both = [&](auto kc) {
+        constexpr int k = decltype(kc)::value, mu = fx::dir_of(k);
+        const char* u = mu == 0 ? fx::links_of_dir(a, r, 0) : a.U + mu * fx::link_bytes(V);
+        const int4* p = fx::at(in, H.nb[k]);
+        const int4* m = fx::at(in, H.nb[k + 1]);
+        fx::half_hop<k, DUAL, fx::kTile, fx::kTile>(H, p + 3 * fx::kTile * f, p + fx::partner(mu, f) * fx::kTile,
+                                                    fx::link_at(u, s), fu, fl, bu, bl);
+        fx::half_hop<k + 1, DUAL, fx::kTile, fx::kTile>(H, m + 3 * fx::kTile * f, m + fx::partner(mu, f) * fx::kTile,
+                                                        fx::link_at(u, H.nb[k + 1]), fu, fl, bu, bl);
+        if constexpr (DUAL && mu == 0) {
+            auto pair_or = [&](uint64_t o) { return o | __shfl_xor_sync(0xffffffffu, o, 16); };
+            int ed = fx::dual_split(H, fu, fl, bu, bl);
+            ed = fx::deriv_scale(H, fu, fl, pair_or(fx::or_bits(fu, fl)), ed);
+            ed = fx::normalise(fu, fl, pair_or(fx::or_bits(fu, fl)), ed);
+            if (first + (lane & 15) < V) {
+                int4* o = fx::at(a.out2 + off, s);
+                fx::store_spin(o, f, fu);
+                fx::store_spin(o, 3 - f, fl);
+                if (f == 0) *fx::exponent_at(a.out2 + off, s) = H.bad ? fx::kNanExp : ed;
+            }
+        }
+        const i64 neg = k == 0 ? -(i64)f : 0;  // the y hops' lower spin; the z hops' has its sign already
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            sums[k / 2][6 * f + q][lane & 15] = H.up[q];
+            sums[k / 2][6 * (mu < 2 ? 3 - f : 2 + f) + q][lane & 15] = mu < 2 ? (H.oth[q] ^ neg) - neg : H.own[q];
+        }
+    };
+    if (warp == 0) both(std::integral_constant<int, 0>{});
+    else if (warp == 1) both(std::integral_constant<int, 2>{});
+    else if (warp == 2) both(std::integral_constant<int, 4>{});
+    else both(std::integral_constant<int, 6>{});
+    __syncthreads();
+    const int eref = eref_of[j];
+    bool bad = eref > fx::kNanTest;
+    i64 v[3];
+    {
+        const fx::Coef D = a.scale->diag;
+        const int d = fx::align_shift(eref, e0_of[j] + D.e);
+        const i64 half = fx::half_of(d);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const i64 sum = (sums[0][3 * t + q][j] + sums[1][3 * t + q][j]) + (sums[2][3 * t + q][j] + sums[3][3 * t + q][j]);
+            fx::Sum m = fx::start(half);
+            fx::mac(m, D.m, fx::Num{x[q].x, x[q].y});
+            const i64 mass = fx::value(m) >> d;
+            v[q] = t < 4 ? mass - sum : sum - mass;
+        }
+    }
+    int E = eref - 1;
+    if constexpr (EPI) {
+        const int ej = E + a.c0e;
+        E = ej;
+        if (a.v1) E = max(E, fx::term_exp(e1, a.c1));
+        if (a.v2) E = max(E, fx::term_exp(e2, a.c2));
+        if (a.v3) E = max(E, fx::term_exp(e3, a.c3));
+        bad = bad || e1 > fx::kNanTest || e2 > fx::kNanTest || e3 > fx::kNanTest;
+        const int d = fx::align_shift(E, ej);
+        const i64 half = fx::half_of(d);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v[q] = fx::shifted(v[q], d, half);
+        if (a.v1) fx::add_term(v, x1, e1, a.c1, E);
+        if (a.v2) fx::add_term(v, x2, e2, a.c2, E);
+        if (a.v3) fx::add_term(v, x3, e3, a.c3, E);
+    }
+    uint64_t o = 0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) o |= (uint64_t)(v[q] ^ (v[q] >> 63));
+#pragma unroll
+    for (int m = 1; m < 8; m *= 2) o |= __shfl_xor_sync(0xffffffffu, o, m);
+    E = fx::normalise(v, o, E);
+    if (first + j < V) {
+        char* out = a.out + off;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const fx::Num z = fx::split(v[q]);
+            *const_cast<int2*>(number(out, q)) = make_int2(z.hi, z.lo);
+        }
+        if (t == 0) *fx::exponent_at(out, sj) = bad ? fx::kNanExp : E;
     }
 }
 
@@ -467,6 +593,19 @@ void launch_fx_dslash(const Geom& g, const FxLinks& U, const void* in, void* out
     for (int k = 0; k < 3; ++k) a.div[k] = fx::make_div((uint32_t)g.L[k]);
     a.V = g.V;
     const bool epi = e.v1 || e.v2 || e.v3 || e.half;
+    const i64 split_blocks = (i64)((g.V + 15) / 16) * nrhs;
+    if (split_blocks <= kSplitBlocks) {
+        const dim3 grid((g.V + 15) / 16, nrhs);
+        if (out_deriv) {
+            if (epi) fx_split_kernel<true, true><<<grid, 128, 0, s>>>(a);
+            else fx_split_kernel<false, true><<<grid, 128, 0, s>>>(a);
+        } else {
+            if (epi) fx_split_kernel<true, false><<<grid, 128, 0, s>>>(a);
+            else fx_split_kernel<false, false><<<grid, 128, 0, s>>>(a);
+        }
+        count_launch();
+        return;
+    }
     int threads = FX_THREADS;
     while (threads > 32 && 2LL * g.V * nrhs < 152LL * 2 * threads) threads /= 2;
     int by = (shape & kShapeRhsMask) > 0 ? (shape & kShapeRhsMask) : 4;

@@ -222,6 +222,14 @@ FX_FN int normalise(i64 (&a)[6], i64 (&b)[6], uint64_t o, int e) {
     return e + sh;
 }
 
+// The same for three of a site's numbers.
+FX_FN int normalise(i64 (&a)[3], uint64_t o, int e) {
+    const int sh = bit_length(o) - kBits;
+    FX_UNROLL
+    for (int k = 0; k < 3; ++k) a[k] = sh > 0 ? shifted(a[k], sh, half_of(sh)) : (i64)((uint64_t)a[k] << -sh);
+    return o == 0 ? kZeroExp : e + sh;
+}
+
 // Three components from `spin` of the site whose component 0 is at b.
 FX_FN void store_spin(int4* b, int spin, const i64 (&a)[6]) {
     FX_UNROLL
@@ -257,6 +265,23 @@ FX_FN void add_term(i64 (&a)[6], const int4 (&v)[3], int e, const Coef& c, int E
             mac(i, c.m, z.im);
             a[2 * k] += value(r) >> d;
             a[2 * k + 1] += value(i) >> d;
+        }
+    }
+}
+
+// The same for three numbers v of one exponent.
+FX_FN void add_term(i64 (&a)[3], const int2 (&v)[3], int e, const Coef& c, int E) {
+    const int d = align_shift(E, term_exp(e, c));
+    const i64 half = half_of(d);
+    FX_UNROLL
+    for (int k = 0; k < 3; ++k) {
+        if (c.unit) {
+            const i64 r = ((i64)v[k].x << (kLimb + 2)) + ((i64)v[k].y << 2);
+            a[k] += shifted(c.unit > 0 ? r : -r, d, half);
+        } else {
+            Sum s = start(half);
+            mac(s, c.m, Num{v[k].x, v[k].y});
+            a[k] += value(s) >> d;
         }
     }
 }
