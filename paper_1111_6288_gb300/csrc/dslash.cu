@@ -257,20 +257,11 @@ struct Args {
     int g5;
 };
 
-// Add one hop in direction MU from the neighbour spinor p through the link u to acc = ch gamma5 (sum of hops),
-// ch = -c_op / 2: forward (FWD) uses U_mu(n) psi(n+mu) with (1 - gamma_mu); backward uses U_mu(n-mu)^+ psi(n-mu)
-// with (1 + gamma_mu).  Everything that scales the hop (ch, the boundary factor, FP16's site scale) is in fac,
-// which the accumulation multiplies by at no cost; only a field's phase on x hops (CPLX) takes a product
-// of its own.  Against scaling each spinor, each hop and the sum this saves 120 of some 1700 instructions a
-// site in FP32 (16^3 x 32 11.45 -> 11.3 us a launch, 24 vectors of 24^3 x 48 1306 -> 1292 us) and 400 of 2660 in
-// FP16 (12 vectors of 16^3 x 32 131 -> 123 us).
-template <int MU, bool FWD, bool CPLX, typename R, typename NUM>
-__device__ __forceinline__ void hop(const Cx<R> (&u)[3][3], const NUM (&p)[12], R fac, Cx<R> phase,
-                                    Cx<R> (&acc)[12]) {
+// The half spinor of a hop in direction MU: (1 - gamma_mu) (FWD) or (1 + gamma_mu) on the neighbour spinor p.
+template <int MU, bool FWD, typename R, typename NUM>
+__device__ __forceinline__ void project(const NUM (&p)[12], Cx<R> (&h)[2][3]) {
     constexpr int S = FWD ? 2 : 0;  // forward: h = psi_up - G psi_dn (multiply G by -1)
     using G = GBlock<MU>;
-    constexpr int LO0 = conj_code(G::diag ? G::A : G::B) + S + 2, LO1 = conj_code(G::diag ? G::B : G::A) + S + 2;
-    Cx<R> h[2][3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         if constexpr (G::diag) {
@@ -281,6 +272,20 @@ __device__ __forceinline__ void hop(const Cx<R> (&u)[3][3], const NUM (&p)[12], 
             h[1][c] = addu<G::B + S>(p[3 + c], p[6 + c]);
         }
     }
+}
+
+// Add one hop in direction MU from its half spinor h through the link u to acc = ch gamma5 (sum of hops),
+// ch = -c_op / 2: forward (FWD) uses U_mu(n) psi(n+mu), backward U_mu(n-mu)^+ psi(n-mu).  Everything that scales the hop (ch, the boundary factor, FP16's site scale) is in fac,
+// which the accumulation multiplies by at no cost; only a field's phase on x hops (CPLX) takes a product
+// of its own.  Against scaling each spinor, each hop and the sum this saves 120 of some 1700 instructions a
+// site in FP32 (16^3 x 32 11.45 -> 11.3 us a launch, 24 vectors of 24^3 x 48 1306 -> 1292 us) and 400 of 2660 in
+// FP16 (12 vectors of 16^3 x 32 131 -> 123 us).
+template <int MU, bool FWD, bool CPLX, typename R>
+__device__ __forceinline__ void hop(const Cx<R> (&u)[3][3], const Cx<R> (&h)[2][3], R fac, Cx<R> phase,
+                                    Cx<R> (&acc)[12]) {
+    constexpr int S = FWD ? 2 : 0;
+    using G = GBlock<MU>;
+    constexpr int LO0 = conj_code(G::diag ? G::A : G::B) + S + 2, LO1 = conj_code(G::diag ? G::B : G::A) + S + 2;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         Cx<R> w[2];
@@ -367,14 +372,14 @@ struct TileSrc {
 // slot_f / slot_b).  XCPLX: the x hops carry the complex factor ph (forward) and conj(ph)
 // (backward).  FP64 links carry the boundary signs (folded in when they are packed), so FP64
 // hops are scaled only by a phase; Dirichlet hops are skipped in both precisions.
-template <typename ST, int MU, bool XCPLX, typename SRC, typename R = typename Arith<ST>::type>
+template <typename ST, int MU, bool XCPLX, bool LATE, typename SRC, typename R = typename Arith<ST>::type>
 __device__ __forceinline__ void both_hops(const Args<R>& a, const SRC& src, int s, int xmu, int slot_f, int slot_b,
                                           Cx<R> ph, Cx<R> (&acc)[12]) {
     constexpr bool FOLD = sizeof(R) == sizeof(double), CPLX = MU == 0 && XCPLX;
     const int L = a.L[MU], st = a.stride[MU];
     const R ch = R(-0.5) * a.c_op;
     typename IO<ST>::Num p[12];
-    Cx<R> u[3][3];
+    Cx<R> u[3][3], h[2][3];
     // forward neighbour
     {
         const bool edge = xmu == L - 1;
@@ -382,8 +387,10 @@ __device__ __forceinline__ void both_hops(const Args<R>& a, const SRC& src, int 
         const R f = edge ? a.bcf[MU] : R(1);
         if (f != R(0)) {
             const R scale = src.load(nb, slot_f, p);
-            IO<ST>::link(a.U, a.V, MU, s, u);
-            hop<MU, true, CPLX>(u, p, (FOLD ? ch : f * ch) * scale, ph, acc);
+            if constexpr (!LATE) IO<ST>::link(a.U, a.V, MU, s, u);
+            project<MU, true>(p, h);
+            if constexpr (LATE) IO<ST>::link(a.U, a.V, MU, s, u);
+            hop<MU, true, CPLX>(u, h, (FOLD ? ch : f * ch) * scale, ph, acc);
         }
     }
     // backward neighbour
@@ -393,8 +400,10 @@ __device__ __forceinline__ void both_hops(const Args<R>& a, const SRC& src, int 
         const R f = edge ? a.bcf[MU] : R(1);
         if (f != R(0)) {
             const R scale = src.load(nb, slot_b, p);
-            IO<ST>::link(a.U, a.V, MU, nb, u);
-            hop<MU, false, CPLX>(u, p, (FOLD ? ch : f * ch) * scale, cconj(ph), acc);
+            if constexpr (!LATE) IO<ST>::link(a.U, a.V, MU, nb, u);
+            project<MU, false>(p, h);
+            if constexpr (LATE) IO<ST>::link(a.U, a.V, MU, nb, u);
+            hop<MU, false, CPLX>(u, h, (FOLD ? ch : f * ch) * scale, cconj(ph), acc);
         }
     }
 }
@@ -568,6 +577,12 @@ template <> struct MinBlocks<double> {
 template <> struct MinBlocks<H16> : MinBlocks<float> {};
 template <> struct MinBlocks<B16> : MinBlocks<float> {};
 
+// A hop's link is loaded after its neighbour is projected where registers allow six blocks an SM, before where
+// they allow seven: late / early, one system of 8^3 x 16 4.46 / 4.55 us and 12 systems 8.84 / 9.10 us a launch with
+// six, 24 systems of 24^3 x 48 1412 / 1328 us with seven.
+template <typename ST, int MINB>
+constexpr bool link_late = MINB == MinBlocks<ST>::value;
+
 // DERIV: instead of H_w, its derivative with respect to the field phase phi of the
 // right-hand side: only the x hops depend on phi, through exp(i phi t) U_x(n) (forward)
 // and exp(-i phi t) U_x(n-x)^+ (backward), whose derivatives bring the factors i t and
@@ -577,6 +592,7 @@ template <> struct MinBlocks<B16> : MinBlocks<float> {};
 template <typename ST, bool DERIV, int MINB>
 __global__ void __launch_bounds__(DSLASH_THREADS, MINB) dslash_kernel(Args<typename Arith<ST>::type> a, int nrhs) {
     using R = typename Arith<ST>::type;
+    constexpr bool LATE = link_late<ST, MINB>;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     const int r = blockIdx.y * blockDim.y + threadIdx.y;
     if (s >= a.V || r >= nrhs) return;
@@ -598,13 +614,13 @@ __global__ void __launch_bounds__(DSLASH_THREADS, MINB) dslash_kernel(Args<typen
     R scale = R(1);
     if constexpr (DERIV) {
         const R tt = (R)x3;
-        both_hops<ST, 0, true>(a, src, s, x0, 0, 0, Cx<R>{-tt * ph.im, tt * ph.re}, acc);  // i t exp(i phi t)
+        both_hops<ST, 0, true, LATE>(a, src, s, x0, 0, 0, Cx<R>{-tt * ph.im, tt * ph.re}, acc);  // i t exp(i phi t)
     } else {
-        both_hops<ST, 2, false>(a, src, s, x2, 0, 0, ph, acc);
-        both_hops<ST, 3, false>(a, src, s, x3, 0, 0, ph, acc);
-        if (a.phase) both_hops<ST, 0, true>(a, src, s, x0, 0, 0, ph, acc);
-        else both_hops<ST, 0, false>(a, src, s, x0, 0, 0, ph, acc);
-        both_hops<ST, 1, false>(a, src, s, x1, 0, 0, ph, acc);
+        both_hops<ST, 2, false, LATE>(a, src, s, x2, 0, 0, ph, acc);
+        both_hops<ST, 3, false, LATE>(a, src, s, x3, 0, 0, ph, acc);
+        if (a.phase) both_hops<ST, 0, true, LATE>(a, src, s, x0, 0, 0, ph, acc);
+        else both_hops<ST, 0, false, LATE>(a, src, s, x0, 0, 0, ph, acc);
+        both_hops<ST, 1, false, LATE>(a, src, s, x1, 0, 0, ph, acc);
         scale = src.load(s, 0, psi);
     }
     finish<ST, DERIV>(a, s, r, psi, scale, acc);
@@ -680,11 +696,11 @@ __global__ void __launch_bounds__(DSLASH_THREADS, MINB) wilson_abi_kernel(Args<t
 #pragma unroll
         for (int k = 0; k < 12; ++k) acc[k] = {R(0), R(0)};
         auto hops = [&](const auto& src) {
-            both_hops<ST, 2, false>(a, src, s, x2, 0, 0, ph, acc);
-            both_hops<ST, 3, false>(a, src, s, x3, 0, 0, ph, acc);
-            if (a.phase) both_hops<ST, 0, true>(a, src, s, x0, 0, 0, ph, acc);
-            else both_hops<ST, 0, false>(a, src, s, x0, 0, 0, ph, acc);
-            both_hops<ST, 1, false>(a, src, s, x1, 0, 0, ph, acc);
+            both_hops<ST, 2, false, false>(a, src, s, x2, 0, 0, ph, acc);
+            both_hops<ST, 3, false, false>(a, src, s, x3, 0, 0, ph, acc);
+            if (a.phase) both_hops<ST, 0, true, false>(a, src, s, x0, 0, 0, ph, acc);
+            else both_hops<ST, 0, false, false>(a, src, s, x0, 0, 0, ph, acc);
+            both_hops<ST, 1, false, false>(a, src, s, x1, 0, 0, ph, acc);
             scale = src.load(s, 0, psi);
         };
         if constexpr (F64) hops(AbiSrc{(const double2*)a.in + (long long)r * 12 * V});
@@ -868,8 +884,8 @@ __global__ void __launch_bounds__(DSLASH_THREADS, MINB) dslash_tiled_kernel(Args
     Cx<R> acc[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] = {R(0), R(0)};
-    both_hops<ST, 2, false>(a, gsrc, s, x2, 0, 0, ph, acc);
-    both_hops<ST, 3, false>(a, gsrc, s, x3, 0, 0, ph, acc);
+    both_hops<ST, 2, false, false>(a, gsrc, s, x2, 0, 0, ph, acc);
+    both_hops<ST, 3, false, false>(a, gsrc, s, x3, 0, 0, ph, acc);
     if (!mbar_wait_bounded(bar_a, 0)) {
         atomicExch(&g_wait_timeouts, 1);
         mbar_wait_bounded(bar_a, 0);
@@ -878,9 +894,9 @@ __global__ void __launch_bounds__(DSLASH_THREADS, MINB) dslash_tiled_kernel(Args
     const TileSrc<ST> tsrc{tiles + threadIdx.y * tile_bytes, P};
     const int slot = L0 + threadIdx.x, row0 = slot - x0;  // this site's slot; slot of x = 0 in its row
     const int xf = row0 + (x0 + 1 == L0 ? 0 : x0 + 1), xb = row0 + (x0 == 0 ? L0 - 1 : x0 - 1);
-    if (a.phase) both_hops<ST, 0, true>(a, tsrc, s, x0, xf, xb, ph, acc);
-    else both_hops<ST, 0, false>(a, tsrc, s, x0, xf, xb, ph, acc);
-    both_hops<ST, 1, false>(a, tsrc, s, x1, slot + L0, slot - L0, ph, acc);
+    if (a.phase) both_hops<ST, 0, true, false>(a, tsrc, s, x0, xf, xb, ph, acc);
+    else both_hops<ST, 0, false, false>(a, tsrc, s, x0, xf, xb, ph, acc);
+    both_hops<ST, 1, false, false>(a, tsrc, s, x1, slot + L0, slot - L0, ph, acc);
     typename IO<ST>::Num psi[12];
     const R scale = tsrc.load(s, slot, psi);
     finish<ST, false>(a, s, r, psi, scale, acc);
