@@ -190,6 +190,7 @@ size_t vec_bytes(const ov_ctx* c, int prec) {
     return (size_t)12 * c->g.V * (prec == OV_PREC_F64 ? 16 : 8);
 }
 double site_spinor_bytes(int prec) { return prec == OV_PREC_F64 ? 196 : prec == OV_PREC_F32 ? 96 : prec == OV_PREC_F16 ? 52 : 48; }
+// (16 bits: of two rows, which a link cannot do without; the third is stored for its instructions)
 double site_link_bytes(int prec) { return prec == OV_PREC_F64 ? 576 : prec == OV_PREC_F32 ? 192 : 96; }
 
 

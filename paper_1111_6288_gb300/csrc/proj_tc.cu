@@ -17,7 +17,7 @@
 // shared memory by TMA (cp.async.bulk.tensor, this GPU's memory, no multicast) through a multi-stage
 // mbarrier pipeline; eight warps split each tile into the hi/lo operand tiles (128-byte swizzled,
 // K-major: one 128-byte row of 32 floats per matrix row); one thread issues tcgen05.mma (kind::tf32,
-// M = 128, cta_group::1) into TMEM accumulators, which the eight warps read back with tcgen05.ld.
+// M = 128, cta_group::1) into TMEM accumulators, which four more warps read back with tcgen05.ld.
 // Every wait on a barrier is bounded (about a second); a wait that runs out records the timeout in
 // g_tc_timeouts and makes every role of the block stop; the block then waits (bounded) for the copies
 // and MMAs it started and frees its TMEM before it returns.
@@ -218,10 +218,10 @@ struct VdotLayout {
 
 // Warp 0 TMA, warp 1 MMA and TMEM, warps 2-9 transform (two warps per scheduler hide each other's
 // shared-memory and conversion latency), warps 10-13 read the accumulators (warp w has TMEM lanes
-// 32 (w % 4) ..).  With the transform warps reading them too, the transform stood still meanwhile: 24
-// vectors on 100 modes of 16^3 x 32 took 1.69 ms for both kernels then and 0.92 ms now (1.05 ms before a_hi met
-// b_hi and b_lo in one MMA, which halves the reads of a_hi); DRAM 3-4 TB/s, bound by shared memory (raw tile
-// in, operand tiles out, MMA reads: about 1100 of 1300 clocks a K-tile) and the conversions (490 clocks).
+// 32 (w % 4) ..).  With the transform warps reading them too, the transform stood still meanwhile: a whole
+// projection of 24 vectors on 100 modes of 16^3 x 32 took 2.0 ms then, 1.35 ms with these warps, and takes 1.22 ms
+// since a_hi meets b_hi and b_lo in one MMA, which halves the reads of a_hi.  By the bytes it is bound by shared
+// memory: raw tile in, operand tiles out, MMA reads.
 constexpr int WS_THREADS = 448;
 constexpr int NXW = 8;                 // transform warps
 constexpr int NXT = NXW * 32;          // transform threads
