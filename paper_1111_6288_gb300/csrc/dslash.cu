@@ -275,10 +275,10 @@ __device__ __forceinline__ void project(const NUM (&p)[12], Cx<R> (&h)[2][3]) {
 }
 
 // Add one hop in direction MU from its half spinor h through the link u to acc = ch gamma5 (sum of hops),
-// ch = -c_op / 2: forward (FWD) uses U_mu(n) psi(n+mu), backward U_mu(n-mu)^+ psi(n-mu).  Everything that scales the hop (ch, the boundary factor, FP16's site scale) is in fac,
-// which the accumulation multiplies by at no cost; only a field's phase on x hops (CPLX) takes a product
-// of its own.  Against scaling each spinor, each hop and the sum this saves 120 of some 1700 instructions a
-// site in FP32 (16^3 x 32 11.45 -> 11.3 us a launch, 24 vectors of 24^3 x 48 1306 -> 1292 us) and more in
+// ch = -c_op / 2: forward (FWD) uses U_mu(n) psi(n+mu), backward U_mu(n-mu)^+ psi(n-mu).  Everything that scales
+// the hop (ch, the boundary factor, FP16's site scale) is in fac, which the accumulation multiplies by at no
+// cost; only a field's phase on x hops (CPLX) takes a product of its own.  Against scaling each spinor, each hop
+// and the sum this saves 120 of some 1700 instructions a site in FP32 (16^3 x 32 11.45 -> 11.3 us a launch, 24 vectors of 24^3 x 48 1306 -> 1292 us) and more in
 // FP16 (12 vectors of 16^3 x 32 131 -> 123 us; with its sums of 16-bit numbers and its third rows 2360 -> 1970
 // instructions a site, 106 us).
 template <int MU, bool FWD, bool CPLX, typename R>

@@ -207,8 +207,8 @@ __global__ void __launch_bounds__(FX_THREADS, kBlocksPerSm) fx_dslash_kernel(con
 
 // The same on few sites, eight lanes a site: there a launch takes as long as one warp's instructions, one
 // every four to five cycles, whatever the memory does (a ring that holds every step took 6.1 us on 4^4 instead
-// of 6.4).  4^4: 6.6 -> 5.1 us.  A block has 16 sites; each of its four warps does the two hops of one direction, operands loaded
-// straight into registers, and the sums meet in shared memory, where each thread takes three of a site's 24
+// of 6.4).  4^4: 6.6 -> 5.1 us.  A block has 16 sites; each of its four warps does the two hops of one direction,
+// operands loaded straight into registers, and the sums meet in shared memory, where each thread takes three of a site's 24
 // numbers through the epilogue.  The sums are integers, so the bits are those of fx_dslash_kernel.
 template <bool EPI, bool DUAL>
 __global__ void __launch_bounds__(128) fx_split_kernel(const __grid_constant__ fx::Args a) {
@@ -220,7 +220,10 @@ __global__ void __launch_bounds__(128) fx_split_kernel(const __grid_constant__ f
     const char* in = a.in + off;
     // numbers 3 t .. 3 t + 2 of site first + j
     const int j = threadIdx.x >> 3, t = threadIdx.x & 7, sj = min(first + j, V - 1);
-    auto number = [&](const char* v, int q) { return (const int2*)(fx::at(v, sj) + ((3 * t + q) >> 1) * fx::kTile) + ((3 * t + q) & 1); };
+    auto number = [&](const char* v, int q) {
+        const int k = 3 * t + q;
+        return (const int2*)(fx::at(v, sj) + (k >> 1) * fx::kTile) + (k & 1);
+    };
     int2 x[3], x1[3], x2[3], x3[3];
     int e1 = 0, e2 = 0, e3 = 0;
     auto fetch = [&](const char* v, int2(&d)[3]) {
@@ -286,7 +289,8 @@ __global__ void __launch_bounds__(128) fx_split_kernel(const __grid_constant__ f
         const i64 half = fx::half_of(d);
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const i64 sum = (sums[0][3 * t + q][j] + sums[1][3 * t + q][j]) + (sums[2][3 * t + q][j] + sums[3][3 * t + q][j]);
+            const int k = 3 * t + q;
+            const i64 sum = (sums[0][k][j] + sums[1][k][j]) + (sums[2][k][j] + sums[3][k][j]);
             fx::Sum m = fx::start(half);
             fx::mac(m, D.m, fx::Num{x[q].x, x[q].y});
             const i64 mass = fx::value(m) >> d;
