@@ -209,8 +209,9 @@ int ov_set_gauge(ov_ctx* ctx, const void* U, int dtype, ov_stream_t stream);
  * x^{-1/2} on [eps, 1] at the n + 1 Chebyshev-Gauss nodes (Sec. 2). out: host [n+1]. */
 int ov_chebyshev_coeffs(int n, double eps, double* out);
 
-/* Eigen-decomposition of a small Hermitian matrix on the host (cyclic Jacobi), the
- * routine the library uses for its Rayleigh-Ritz and Gram matrices.  A: host, n x n
+/* Eigen-decomposition of a small Hermitian matrix on the host (tridiagonalisation and implicit QR),
+ * the routine the library uses for its Rayleigh-Ritz and Gram matrices (NaN for a matrix that is not
+ * finite; OV_ERR_NOT_CONVERGED if the QR steps did not converge).  A: host, n x n
  * column-major complex128 (overwritten); w: host [n] eigenvalues ascending; Z: host
  * n x n column-major complex128 eigenvectors (A = Z diag(w) Z^+).  No GPU needed. */
 int ov_host_eigh(int n, double* A, double* w, double* Z);

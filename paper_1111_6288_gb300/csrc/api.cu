@@ -1065,7 +1065,7 @@ int eig_rayleigh_ritz(ov_ctx* c, int m, int n_ev, void*& W, void*& W2, void*& QW
         std::vector<double> mu;
         TRY(gram_host<R>(c, QW, m, QW, m, G2, s));
         hermitize(G2, m);
-        host_eigh(m, G2, mu, Y);
+        if (!host_eigh(m, G2, mu, Y)) return fail(c, OV_ERR_NAN, "Rayleigh-Ritz: eigenproblem of Q^2 not solved");
         a = std::min(mu[m - 1], 0.95);
         void* const w_old = W;
         void* const qw_old = QW;
@@ -1079,7 +1079,7 @@ int eig_rayleigh_ritz(ov_ctx* c, int m, int n_ev, void*& W, void*& W2, void*& QW
     TRY(gram_host<R>(c, W, n_ev, QW, n_ev, T, s));
     hermitize(T, n_ev);
     std::vector<double> w;
-    host_eigh(n_ev, T, w, Z);
+    if (!host_eigh(n_ev, T, w, Z)) return fail(c, OV_ERR_NAN, "Rayleigh-Ritz: eigenproblem of Q not solved");
     std::vector<int> order(n_ev);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int i, int j) {
@@ -1257,7 +1257,8 @@ int ov_host_eigh(int n, double* A, double* w, double* Z) {
     std::vector<HostCplx> M((size_t)n * n), Zm;
     std::memcpy(M.data(), A, sizeof(HostCplx) * n * n);
     std::vector<double> wv;
-    host_eigh(n, M, wv, Zm);
+    // w is NaN for a matrix that is not finite
+    if (!host_eigh(n, M, wv, Zm) && !std::isnan(wv[0])) return OV_ERR_NOT_CONVERGED;
     std::memcpy(w, wv.data(), sizeof(double) * n);
     std::memcpy(Z, Zm.data(), sizeof(HostCplx) * n * n);
     return OV_OK;
@@ -1809,7 +1810,7 @@ int lanczos_overlap(ov_ctx* c, double phase, int chi, int n_ev, int K, double to
                 T[j + (size_t)i * K] = HostCplx{h.re, -h.im};
             }
         }
-        host_eigh(K, T, th, Y);
+        if (!host_eigh(K, T, th, Y)) return fail(c, OV_ERR_NAN, "D_ov Lanczos: projected eigenproblem not solved");
         worst_est = 0.0;
         for (int i = 0; i < n_ev; ++i) {
             const HostCplx y = Y[(K - 1) + (size_t)i * K];
@@ -1859,7 +1860,7 @@ int lanczos_overlap(ov_ctx* c, double phase, int chi, int n_ev, int K, double to
     std::vector<HostCplx> Hr, Z;
     TRY(gram_host<float>(c, sp->W, n_ev, sp->AW0, n_ev, Hr, s));
     hermitize(Hr, n_ev);
-    host_eigh(n_ev, Hr, sp->theta, Z);
+    if (!host_eigh(n_ev, Hr, sp->theta, Z)) return fail(c, OV_ERR_NAN, "D_ov low modes: eigenproblem not solved");
     TRY(rotate<float>(c, sp->W, n_ev, Z, n_ev, tmp, s));
     CK(cudaMemcpyAsync(sp->W, tmp, vb * n_ev, cudaMemcpyDeviceToDevice, s));
     TRY(rotate<float>(c, sp->AW0, n_ev, Z, n_ev, tmp, s));

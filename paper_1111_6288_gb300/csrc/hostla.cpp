@@ -6,6 +6,7 @@
 // Matrices are column-major arrays of (re, im) pairs, A(i, j) = A[i + j n].
 #include <algorithm>
 #include <cmath>
+#include <limits>
 #include <numeric>
 #include <vector>
 
@@ -75,15 +76,25 @@ void tridiagonalise(int n, std::vector<HostCplx>& A, std::vector<double>& d, std
     for (int k = 0; k + 1 < n; ++k) {
         const int m = n - k - 1, r0 = k + 1;
         HostCplx* v = &A[r0 + (size_t)k * n];
-        double below = 0.0;
-        for (int i = 1; i < m; ++i) below += norm(v[i]);
-        const HostCplx a = v[0];
         d[k] = A[k + (size_t)k * n].re;
-        if (below == 0.0 && a.im == 0.0) {  // already real: no reflection
-            e[k] = a.re;
+        double rest = 0.0;
+        for (int i = 1; i < m; ++i) rest = std::max(rest, std::max(std::fabs(v[i].re), std::fabs(v[i].im)));
+        const double most = std::max(rest, std::max(std::fabs(v[0].re), std::fabs(v[0].im)));
+        if (rest == 0.0 && v[0].im == 0.0) {  // already real: no reflection
+            e[k] = v[0].re;
             tau[k] = HostCplx{0.0, 0.0};
             continue;
         }
+        // The column's largest number is brought near 1: a column may be far below the matrix, and its squares
+        // below the smallest double.
+        int scale = 0;
+        std::frexp(most, &scale);
+        double below = 0.0;
+        for (int i = 0; i < m; ++i) {
+            v[i] = HostCplx{std::ldexp(v[i].re, -scale), std::ldexp(v[i].im, -scale)};
+            if (i > 0) below += norm(v[i]);
+        }
+        const HostCplx a = v[0];
         const double beta = -std::copysign(std::sqrt(norm(a) + below), a.re);
         tau[k] = HostCplx{(beta - a.re) / beta, -a.im / beta};
         const HostCplx t{a.re - beta, a.im};  // v = (x - beta e_1) / (a - beta)
@@ -91,7 +102,7 @@ void tridiagonalise(int n, std::vector<HostCplx>& A, std::vector<double>& d, std
         const HostCplx inv{t.re * q, -t.im * q};
         for (int i = 1; i < m; ++i) v[i] = inv * v[i];
         v[0] = HostCplx{1.0, 0.0};
-        e[k] = beta;
+        e[k] = std::ldexp(beta, scale);
         // w = tau A v - 1/2 tau (tau A v, v) v on the trailing block
         std::fill(w.begin(), w.begin() + m, HostCplx{0.0, 0.0});
         for (int j = 0; j < m; ++j) subtract(m, HostCplx{-v[j].re, -v[j].im}, &A[r0 + (size_t)(r0 + j) * n], w.data());
@@ -115,8 +126,8 @@ void tridiagonalise(int n, std::vector<HostCplx>& A, std::vector<double>& d, std
 
 // Eigenvalues of the tridiagonal (d, e) into d, the rotations accumulated into Z (n x n, column-major):
 // implicit QR steps with Wilkinson's shift on unreduced blocks (Golub and Van Loan, Matrix
-// Computations, section 8.3).
-void diagonalise(int n, std::vector<double>& d, std::vector<double>& e, std::vector<double>& Z) {
+// Computations, section 8.3).  false: not converged.
+bool diagonalise(int n, std::vector<double>& d, std::vector<double>& e, std::vector<double>& Z) {
     const double eps = 2.220446049250313e-16, floor = 1e-280;  // (the largest number is near 1)
     int hi = n - 1;
     for (int steps = 0; hi > 0 && steps < 60 * n; ++steps) {
@@ -151,20 +162,31 @@ void diagonalise(int n, std::vector<double>& d, std::vector<double>& e, std::vec
             }
         }
     }
+    return hi == 0;
 }
 }  // namespace
 
-void host_eigh(int n, std::vector<HostCplx>& A, std::vector<double>& w, std::vector<HostCplx>& Z) {
+bool host_eigh(int n, std::vector<HostCplx>& A, std::vector<double>& w, std::vector<HostCplx>& Z) {
     // Reflections to real tridiagonal form, its eigenvectors by QR steps, and the reflections applied to
     // them.  32 x 32: 0.4 ms where cyclic Jacobi sweeps took 9; 256 x 256: 0.12 against 5.2 s.
     w.assign(n, 0.0);
     Z.assign((size_t)n * n, HostCplx{0.0, 0.0});
-    if (n < 1) return;
-    // the largest number is brought near 1, so that no square over- or underflows
+    if (n < 1) return true;
+    // the largest number is brought near 1, so that no square overflows
     double most = 0.0;
-    for (const HostCplx& v : A) most = std::max(most, std::max(std::fabs(v.re), std::fabs(v.im)));
+    bool finite = true;
+    for (const HostCplx& v : A) {
+        finite = finite && std::isfinite(v.re) && std::isfinite(v.im);
+        most = std::max(most, std::max(std::fabs(v.re), std::fabs(v.im)));
+    }
+    if (!finite) {
+        const double nan = std::numeric_limits<double>::quiet_NaN();
+        w.assign(n, nan);
+        Z.assign((size_t)n * n, HostCplx{nan, nan});
+        return false;
+    }
     int scale = 0;
-    if (most > 0.0 && std::isfinite(most)) {
+    if (most > 0.0) {
         std::frexp(most, &scale);
         for (HostCplx& v : A) v = HostCplx{std::ldexp(v.re, -scale), std::ldexp(v.im, -scale)};
     }
@@ -172,7 +194,7 @@ void host_eigh(int n, std::vector<HostCplx>& A, std::vector<double>& w, std::vec
     std::vector<HostCplx> tau(n, HostCplx{0.0, 0.0});
     tridiagonalise(n, A, d, e, tau);
     for (int i = 0; i < n; ++i) Y[i + (size_t)i * n] = 1.0;
-    diagonalise(n, d, e, Y);
+    const bool converged = diagonalise(n, d, e, Y);
     std::vector<int> order(n);
     std::iota(order.begin(), order.end(), 0);
     std::sort(order.begin(), order.end(), [&](int a, int b) { return d[a] < d[b]; });
@@ -191,6 +213,7 @@ void host_eigh(int n, std::vector<HostCplx>& A, std::vector<double>& w, std::vec
             subtract(n - k - 1, tau[k] * dot, v, z + k + 1);
         }
     }
+    return converged;
 }
 
 namespace {

@@ -219,9 +219,10 @@ struct HostCplx { double re, im; };
 bool host_cholesky(int n, std::vector<HostCplx>& A);
 // Inverse of the conjugate transpose of a lower-triangular L: returns R = L^{-+} (upper).
 void host_inv_lower_dag(int n, const std::vector<HostCplx>& L, std::vector<HostCplx>& R);
-// Eigen-decomposition of a Hermitian matrix (cyclic Jacobi): A = Z diag(w) Z^+,
-// eigenvalues ascending. A is overwritten.
-void host_eigh(int n, std::vector<HostCplx>& A, std::vector<double>& w, std::vector<HostCplx>& Z);
+// Eigen-decomposition of a Hermitian matrix (tridiagonalisation and implicit QR): A = Z diag(w) Z^+,
+// eigenvalues ascending. A is overwritten.  false: A is not finite (w and Z are NaN), or the QR steps did
+// not converge.
+bool host_eigh(int n, std::vector<HostCplx>& A, std::vector<double>& w, std::vector<HostCplx>& Z);
 // Chebyshev interpolant coefficients of x^{-1/2} on [eps, 1] (c_0 halved).
 void host_chebyshev_coeffs(int n, double eps, double* out);
 // The same for 1/(a + sqrt(x)), a > 0.

@@ -2,6 +2,8 @@
 wrong: 1 x 1, 2 x 2, matrices that split (diagonal, blocks, zero), many equal eigenvalues, entries near the
 ends of the exponent range.
 
+Couplings far below the matrix's largest entry, whose squares underflow, are one more.
+
 Tolerance: a backward stable method is off by a small multiple of n 2^-53 |A|; 16 n of them are allowed, for
 the eigenvalues, the residuals and the orthogonality (|A| the largest eigenvalue).
 """
@@ -45,3 +47,37 @@ def test_host_eigh(kind, n, scale):
     assert np.all(np.diff(w) >= 0)
     assert np.abs(Z.conj().T @ Z - np.eye(n)).max() <= tol
     assert np.abs(A @ Z - Z * (w / scale)).max() <= tol * norm
+
+
+@pytest.mark.parametrize("n", [2, 3, 5])
+@pytest.mark.parametrize("tiny", [1e-155, 1e-160, 1e-165j, 1e-200j, 1e-300 + 1e-310j, 5e-324j])
+@pytest.mark.parametrize("where", ["all", "first", "last"])
+def test_tiny_couplings(n, tiny, where):
+    """O(1) diagonals with couplings whose squares underflow: all of them, or one beside ordinary ones."""
+    import paper_1111_6288_gb300 as P
+
+    A = np.diag(1.0 + np.arange(n)).astype(complex)
+    low = np.tril(np.ones((n, n)), -1) * tiny
+    if where != "all" and n > 2:
+        low = np.tril(0.1 * np.ones((n, n)), -1).astype(complex)
+        low[(1, 0) if where == "first" else (n - 1, 0)] = tiny
+        if where == "first":
+            low[2:, 0] = 0
+    A += low + low.conj().T
+    w, Z = P.host_eigh(A)
+    want = np.linalg.eigvalsh(A)
+    tol = 16 * n * 2.0**-53
+    norm = np.abs(want).max()
+    assert np.abs(w - want).max() <= tol * norm
+    assert np.abs(Z.conj().T @ Z - np.eye(n)).max() <= tol
+    assert np.abs(A @ Z - Z * w).max() <= tol * norm
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, complex(0, np.nan)])
+def test_not_finite(bad):
+    import paper_1111_6288_gb300 as P
+
+    A = np.eye(3, dtype=complex)
+    A[2, 1] = A[1, 2] = bad
+    w, Z = P.host_eigh(A)
+    assert np.isnan(w).all() and np.isnan(Z).all()
