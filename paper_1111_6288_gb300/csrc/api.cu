@@ -451,7 +451,7 @@ int fx_links(ov_ctx* c, const SysSet& S, double scale2, FxLinks* L, cudaStream_t
 
 // The epilogue of a fixed-point application with the same vectors; its links carry the operator's
 // coefficient up to the factor 1/2 of a recurrence's last or first step.
-FxEpilogue fx_epilogue(const Epilogue& e, bool half = false) {
+FxEpilogue fx_epilogue(const Epilogue& e, bool half) {
     FxEpilogue f;
     f.half = half;
     f.c1 = e.c1;
@@ -663,8 +663,9 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
     // the whole recurrence (2n launches, no host work) as one stream sequence
     // timing launches read t, bA, x_perp and write bB only (rewritten by the recurrence below)
     const int nconv = FX ? 3 : (HALF ? 2 : 1);  // launches besides the recurrence
-    auto step = [&](const void* in, void* o, const Epilogue& e, cudaStream_t st, int shape) {
-        if constexpr (FX) launch_fx_dslash(c->g, fxl, in, o, nullptr, ns, fx_epilogue(e, e.c_op == 0.5 * alpha), st, shape);
+    // half: the step's operator is (alpha / 2) H_w^2, which the links of the fixed-point recurrence do not carry
+    auto step = [&](const void* in, void* o, const Epilogue& e, cudaStream_t st, int shape, bool half = false) {
+        if constexpr (FX) launch_fx_dslash(c->g, fxl, in, o, nullptr, ns, fx_epilogue(e, half), st, shape);
         else launch_dslash<ST>(c->g, m0, Us, in, o, ns, d_phase, e, st, false, shape);
     };
     const int rb = tuned_shape<ST>(c, ns, t, bA, xs, bA, bB, s, step);
@@ -693,7 +694,7 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
             e.c3 = -1.0;
             e.v3 = b2;
             void* o = b2 ? b2 : bB;
-            step(t, o, e, st, rb);
+            step(t, o, e, st, rb, k == 0);
             b2 = b1;
             b1 = o;
         }
@@ -1004,8 +1005,8 @@ int cheb_filter(ov_ctx* c, void* W, int m, double a, int degree, const SysSet& S
     if (FX) TRY(fx_links(c, S, 2.0 * za, &fxl, s));
     for (int j0 = 0; j0 < m; j0 += cw) {
         const int nj = std::min(cw, m - j0);
-        auto step = [&](const void* in, void* out, const Epilogue& e) {
-            if constexpr (FX) launch_fx_dslash(c->g, fxl, in, out, nullptr, nj, fx_epilogue(e, e.c_op == za), s, 0);
+        auto step = [&](const void* in, void* out, const Epilogue& e, bool half = false) {
+            if constexpr (FX) launch_fx_dslash(c->g, fxl, in, out, nullptr, nj, fx_epilogue(e, half), s, 0);
             else launch_dslash<R>(c->g, m0, c->U32, in, out, nj, d_phase, e, s);
         };
         void* Wj = (char*)W + vb * j0;
@@ -1017,7 +1018,7 @@ int cheb_filter(ov_ctx* c, void* W, int m, double a, int degree, const SysSet& S
         e1.c_op = za;
         e1.c1 = zb;
         e1.v1 = Tm;
-        step(tt, Tc, e1);  // T_1 = Z W
+        step(tt, Tc, e1, true);  // T_1 = Z W, half of a later step's 2 Z
         void* tk = Tc;
         void* tkm = Tm;
         for (int k = 1; k < degree; ++k) {

@@ -119,3 +119,21 @@ def test_zero_and_nan(P):
         clean[0, 0, 0, 0] = 0.0
         want = oracle_sign(U, clean, bc, hw, degree, 0.0)
         assert np.linalg.norm(y[j, 4:] - want[4:]) <= bound(degree) * np.linalg.norm(want[4:])
+
+
+@pytest.mark.parametrize("hw, eps", [(4.0, 0.875), (2.0, 0.5), (8.0, 0.96875), (4.0, 0.75)])
+@pytest.mark.parametrize("degree", [1, 4])
+def test_operator_coefficients_that_are_powers_of_two(P, hw, eps, degree):
+    """alpha = 4 / ((1 - eps) h^2) of exactly 2 and 1: half of it, or all of it, is the coefficient of a plain
+    step as well.  Only the last step of the recurrence is halved."""
+    dims, bc = (4, 3, 2, 5), (0, 0, 0, 1)
+    assert 4 / ((1 - eps) * hw**2) in (1.0, 2.0)
+    U = synth.random_su3_field(dims, 0.3, seed=21)
+    x = synth.gaussian_spinor(dims, 1, 22)
+    y, _ = run(P, dims, bc, U, x, degree, [0.0], eps=eps, hw=hw)
+    want = oracle_sign(U, x[0], bc, hw, degree, 0.0, eps=eps)
+    # the spectrum of Q^2, [0, (6.5 / hw)^2], leaves [eps, 1] on both sides: T_n of its far ends is the growth
+    ends = (1 + eps) / (1 - eps), (2 * (6.5 / hw) ** 2 - (1 + eps)) / (1 - eps)
+    growth = np.cosh(degree * np.arccosh(max(ends)))
+    assert np.linalg.norm(y[0] - want) <= bound(degree) * growth * np.linalg.norm(x[0])
+    assert np.linalg.norm(want) > 1e3 * bound(degree) * growth * np.linalg.norm(x[0])
