@@ -222,11 +222,12 @@ FX_FN int normalise(i64 (&a)[6], i64 (&b)[6], uint64_t o, int e) {
     return e + sh;
 }
 
-// The same for three of a site's numbers.
+// The same for three of a site's numbers (0 and -1 are nothing here too).
 FX_FN int normalise(i64 (&a)[3], uint64_t o, int e) {
     const int sh = bit_length(o) - kBits;
     FX_UNROLL
-    for (int k = 0; k < 3; ++k) a[k] = sh > 0 ? shifted(a[k], sh, half_of(sh)) : (i64)((uint64_t)a[k] << -sh);
+    for (int k = 0; k < 3; ++k)
+        a[k] = o == 0 ? 0 : sh > 0 ? shifted(a[k], sh, half_of(sh)) : (i64)((uint64_t)a[k] << -sh);
     return o == 0 ? kZeroExp : e + sh;
 }
 

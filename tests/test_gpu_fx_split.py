@@ -12,6 +12,13 @@ pytestmark = pytest.mark.gpu
 BLOCKS = 3 * 152  # of 16 sites, the most that take eight lanes a site
 
 
+def bits(v):
+    """The numbers as integers, so that -0.0 is not 0.0 (NaNs as 0)."""
+    import torch
+
+    return torch.where(torch.isnan(v), torch.zeros_like(v), v).view(torch.int64)
+
+
 @pytest.mark.parametrize("op", ["sign", "overlap", "derivative"])
 @pytest.mark.parametrize("dims", [(2, 2, 4, 4), (3, 3, 3, 3), (5, 3, 4, 7), (4, 4, 4, 4), (8, 8, 6, 5)])
 @pytest.mark.parametrize("bc, phase", [((0, 0, 0, 1), 0.0), ((1, 2, 0, 2), 0.3), ((2, 0, 1, 0), -0.2)])
@@ -50,7 +57,7 @@ def test_alone_and_in_a_batch(dims, bc, phase, op):
     for j in range(3):
         alone = run(x[j : j + 1])[0]
         assert torch.equal(torch.isnan(alone), torch.isnan(batch[j]))
-        assert torch.equal(torch.nan_to_num(alone), torch.nan_to_num(batch[j]))
-    assert torch.equal(torch.nan_to_num(batch[0]), torch.nan_to_num(batch[-1]))
+        assert torch.equal(bits(alone), bits(batch[j]))
+    assert torch.equal(bits(batch[0]), bits(batch[-1]))
     assert not torch.isnan(batch[0]).any()
     ctx.close()
