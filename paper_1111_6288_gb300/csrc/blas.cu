@@ -235,20 +235,30 @@ __global__ void pack_gauge_half_k(const TI* __restrict__ abi, void* __restrict__
 
 constexpr int RT = 256;
 
-// (re, im) += a b, and conj(a) b, four fused multiply-adds (written as sums of products they are six
-// operations: nvcc fuses within a product's sum only)
+// A sum of complex products, each of its four kinds of real products in a sum of its own: four fused
+// multiply-adds a complex product, where a sum of (a.x b.x + a.y b.y) takes six operations (nvcc fuses within
+// a product only).  Each of the four is rounded once a product and is half as large as what it adds up to, so
+// the rounding error is no larger than that of the six.  (Both real products fused into one sum round it twice: errors
+// 1.4 times as large.)
 __device__ __forceinline__ float fmad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmad(double a, double b, double c) { return __fma_rn(a, b, c); }
-template <typename R, typename T>
-__device__ __forceinline__ void mac(R& re, R& im, T a, T b) {
-    re = fmad(-a.y, b.y, fmad(a.x, b.x, re));
-    im = fmad(a.y, b.x, fmad(a.x, b.y, im));
-}
-template <typename R, typename T>
-__device__ __forceinline__ void mac_conj(R& re, R& im, T a, T b) {
-    re = fmad(a.y, b.y, fmad(a.x, b.x, re));
-    im = fmad(-a.y, b.x, fmad(a.x, b.y, im));
-}
+template <typename R>
+struct ProductSum {
+    R xx = 0, yy = 0, xy = 0, yx = 0;
+    template <typename T>
+    __device__ __forceinline__ void add(T a, T b) {
+        xx = fmad(a.x, b.x, xx);
+        yy = fmad(a.y, b.y, yy);
+        xy = fmad(a.x, b.y, xy);
+        yx = fmad(a.y, b.x, yx);
+    }
+    // of a b
+    __device__ __forceinline__ R re() const { return xx - yy; }
+    __device__ __forceinline__ R im() const { return xy + yx; }
+    // of conj(a) b
+    __device__ __forceinline__ double conj_re() const { return (double)xx + (double)yy; }
+    __device__ __forceinline__ double conj_im() const { return (double)xy - (double)yx; }
+};
 
 // s + c += x in FP32, c what the rounding of s leaves (Knuth's two-sum)
 __device__ __forceinline__ void add_exact(float& s, float& c, float x) {
@@ -413,7 +423,7 @@ __global__ void __launch_bounds__(MNT) multidot_k(const typename C2<R>::T* __res
     const int t = threadIdx.x;
     const int pair = t & 63, part = t >> 6;  // 64 (i, j) pairs x 4 parts of a slab
     const int pi = pair >> 3, pj = pair & 7;
-    R sre = 0, sim = 0;
+    ProductSum<R> sum;
     for (long long k0 = k_begin; k0 < k_end; k0 += MK) {
         {
             const int v = t >> 5, e = t & 31;  // 8 vectors x 32 elements
@@ -430,11 +440,11 @@ __global__ void __launch_bounds__(MNT) multidot_k(const typename C2<R>::T* __res
         __syncthreads();
 #pragma unroll
         for (int e = part * 8; e < part * 8 + 8; ++e) {
-            mac_conj(sre, sim, shA[pi][e], shB[pj][e]);
+            sum.add(shA[pi][e], shB[pj][e]);
         }
         __syncthreads();
     }
-    red[t] = make_double2((double)sre, (double)sim);
+    red[t] = make_double2(sum.conj_re(), sum.conj_im());
     __syncthreads();
     if (t < 64) {
         double2 v = red[t];
@@ -452,10 +462,15 @@ __global__ void __launch_bounds__(MNT) multidot_k(const typename C2<R>::T* __res
 __global__ void multidot_sum_k(const double2* __restrict__ partial, int nchunk, int nab, double2* __restrict__ C) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= nab) return;
-    double2 v = make_double2(0, 0);
-#pragma unroll 8
-    for (int c = 0; c < nchunk; ++c) v = dadd(v, partial[(long long)c * nab + idx]);
-    C[idx] = v;
+    // four sums side by side: what they round is a quarter as far apart as in one chain
+    double2 v[4];
+    for (double2& z : v) z = make_double2(0, 0);
+#pragma unroll 2
+    for (int c = 0; c < nchunk; c += 4)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (c + q < nchunk) v[q] = dadd(v[q], partial[(long long)(c + q) * nab + idx]);
+    C[idx] = dadd(dadd(v[0], v[1]), dadd(v[2], v[3]));
 }
 
 // out_j = alpha X_j + sum_i A_i C[i][j], up to CJ outputs per launch; the coefficients are
@@ -477,21 +492,21 @@ __global__ void __launch_bounds__(256) combine_k(const typename C2<R>::T* __rest
     __syncthreads();
     const R al = (R)alpha;
     for (long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x; m < n; m += (long long)gridDim.x * blockDim.x) {
-        R accr[CJT], acci[CJT];
-#pragma unroll
-        for (int j = 0; j < CJT; ++j) accr[j] = acci[j] = 0;
+        ProductSum<R> acc[CJT];
 #pragma unroll 4
         for (int i = 0; i < na; ++i) {
             typename C2<R>::T a = A[(long long)i * sA + m];
 #pragma unroll
             for (int j = 0; j < CJT; ++j) {
-                mac(accr[j], acci[j], a, shC[i * CJT + j]);
+                acc[j].add(a, shC[i * CJT + j]);
             }
         }
-        for (int j = 0; j < nj; ++j) {
+#pragma unroll
+        for (int j = 0; j < CJT; ++j) {
+            if (j >= nj) break;
             typename C2<R>::T o;
-            o.x = accr[j];
-            o.y = acci[j];
+            o.x = acc[j].re();
+            o.y = acc[j].im();
             if (X) {
                 typename C2<R>::T xv = X[(long long)(j0 + j) * sX + m];
                 o.x += al * xv.x;
@@ -504,26 +519,27 @@ __global__ void __launch_bounds__(256) combine_k(const typename C2<R>::T* __rest
 
 // ---- small-space projection for a few right-hand sides ---------------------
 //
-// C[i][j] = <V_i, X_j> for j < nb <= SP_NB: each warp owns 8 rows of V and walks a
+// C[i][j] = <V_i, X_j> for j < nb <= SP_NB: each warp owns some rows of V and walks a
 // chunk of the element range, so every element of V is read once; each lane keeps
-// 8 x nb partial sums (in R), reduced across the warp in a fixed order and written
+// rows x nb partial sums (in R), reduced across the warp in a fixed order and written
 // per chunk (the chunks are added by multidot_sum_k, also in a fixed order).
 constexpr int SP_NB = 4;
-constexpr int SP_ROWS = 8;  // rows per warp; 8 warps -> 64 rows per block
+// Rows per warp (8 warps a block), by the columns: few, so that many warps hide the loads.  V^+ X with 50 rows of
+// 16^3 x 32 in FP32 / FP64, 1, 2 or 4 columns: 264 / 823, 275 / 1519 and 525 / 2567 us; with four times the rows
+// 304 / 846, 535 / 1604 and 695 / 2949 us.
+constexpr int sp_rows(int nb) { return nb > 2 ? 1 : 2; }
+inline unsigned sp_row_blocks(int na, int nb) { return (na + 8 * sp_rows(nb) - 1) / (8 * sp_rows(nb)); }
 
 template <typename R, int NB>
 __global__ void __launch_bounds__(256) vdot_rows_k(const typename C2<R>::T* __restrict__ V, long long sV, int na,
                                                    const typename C2<R>::T* __restrict__ X, long long sX, int nb,
                                                    long long n, long long chunk, double2* __restrict__ partial) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row0 = blockIdx.y * 64 + warp * SP_ROWS;
+    constexpr int ROWS = sp_rows(NB);
+    const int row0 = (blockIdx.y * 8 + warp) * ROWS;
     const long long k_begin = (long long)blockIdx.x * chunk;
     const long long k_end = min(n, k_begin + chunk);
-    R ar[SP_ROWS][NB], ai[SP_ROWS][NB];
-#pragma unroll
-    for (int r = 0; r < SP_ROWS; ++r)
-#pragma unroll
-        for (int j = 0; j < NB; ++j) ar[r][j] = ai[r][j] = 0;
+    ProductSum<R> sum[ROWS][NB];
     for (long long m = k_begin + lane; m < k_end; m += 32) {
         typename C2<R>::T xv[NB];
 #pragma unroll
@@ -532,22 +548,22 @@ __global__ void __launch_bounds__(256) vdot_rows_k(const typename C2<R>::T* __re
             else xv[j].x = xv[j].y = 0;
         }
 #pragma unroll
-        for (int r = 0; r < SP_ROWS; ++r) {
+        for (int r = 0; r < ROWS; ++r) {
             const int i = row0 + r;
             if (i < na) {
                 const typename C2<R>::T v = V[(long long)i * sV + m];
 #pragma unroll
                 for (int j = 0; j < NB; ++j) {  // conj(v) * x
-                    mac_conj(ar[r][j], ai[r][j], v, xv[j]);
+                    sum[r][j].add(v, xv[j]);
                 }
             }
         }
     }
 #pragma unroll
-    for (int r = 0; r < SP_ROWS; ++r)
+    for (int r = 0; r < ROWS; ++r)
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
-            double re = (double)ar[r][j], im = (double)ai[r][j];
+            double re = sum[r][j].conj_re(), im = sum[r][j].conj_im();
             for (int o = 16; o > 0; o >>= 1) {
                 re += __shfl_down_sync(0xffffffffu, re, o);
                 im += __shfl_down_sync(0xffffffffu, im, o);
@@ -578,16 +594,15 @@ __global__ void __launch_bounds__(256) proj_apply_k(const typename C2<R>::T* __r
     }
     __syncthreads();
     for (long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x; m < n; m += (long long)gridDim.x * blockDim.x) {
-        R a1r[NB], a1i[NB], a2r[NB], a2i[NB];
-#pragma unroll
-        for (int j = 0; j < NB; ++j) a1r[j] = a1i[j] = a2r[j] = a2i[j] = 0;
+        ProductSum<R> a1[NB], a2[NB];
+#pragma unroll 8
         for (int i = 0; i < na; ++i) {
             const typename C2<R>::T v = V[(long long)i * sV + m];
 #pragma unroll
             for (int j = 0; j < NB; ++j) {
                 const typename C2<R>::T c1 = cn[i * NB + j], c2 = cs[i * NB + j];
-                mac(a1r[j], a1i[j], v, c1);
-                mac(a2r[j], a2i[j], v, c2);
+                a1[j].add(v, c1);
+                a2[j].add(v, c2);
             }
         }
 #pragma unroll
@@ -595,10 +610,10 @@ __global__ void __launch_bounds__(256) proj_apply_k(const typename C2<R>::T* __r
             if (j < nj) {
                 const long long o = (long long)(j0 + j) * sX + m;
                 typename C2<R>::T xv = X[o], p, y;
-                p.x = xv.x + a1r[j];
-                p.y = xv.y + a1i[j];
-                y.x = a2r[j];
-                y.y = a2i[j];
+                p.x = xv.x + a1[j].re();
+                p.y = xv.y + a1[j].im();
+                y.x = a2[j].re();
+                y.y = a2[j].im();
                 Xp[o] = p;
                 Ys[o] = y;
             }
@@ -763,14 +778,14 @@ template <typename R, int NB>
 void multidot_few(const void* A, long long sA, int na, const void* B, long long sB, int nb, long long n, double2* d_C,
                   double2* d_partial, long long partial_cap, cudaStream_t s) {
     typedef typename C2<R>::T T;
-    const int rowblocks = (na + 63) / 64;
+    const int rowblocks = (na + 63) / 64;  // (the chunks' lengths do not depend on the rows of a warp)
     long long nchunk = std::max((4LL * 152 + rowblocks - 1) / rowblocks, (n + 4095) / 4096);
     const long long cap = partial_cap / ((long long)na * nb);
     if (nchunk > cap) nchunk = std::max(1LL, cap);
     long long chunk = (n + nchunk - 1) / nchunk;
     chunk = ((chunk + 31) / 32) * 32;
     nchunk = (n + chunk - 1) / chunk;
-    dim3 grid((unsigned)nchunk, rowblocks);
+    dim3 grid((unsigned)nchunk, sp_row_blocks(na, NB));
     vdot_rows_k<R, NB><<<grid, 256, 0, s>>>((const T*)A, sA, na, (const T*)B, sB, nb, n, chunk, d_partial);
     count_launch();
     const int nab = na * nb;
@@ -825,8 +840,8 @@ void combine(const void* A, long long strideA, int na, const double2* d_C, int l
         return;
     }
     // FP64: blocks of 64, so that the FP64 pipes of all SMs end together.  8 columns from 32 vectors of
-    // 8^3 x 16: 299 us with 384 blocks of 256 on the 152 SMs and six operations a product, 282 us with blocks of
-    // 64, 171 us with four operations as well, what the FP64 pipe takes for them.
+    // 8^3 x 16: 327 us with 384 blocks of 256 on the 152 SMs and six operations a product, 199 us with blocks of 64
+    // and four operations (187 us with two sums instead of ProductSum's four, which round twice a product).
     constexpr int NT = std::is_same<R, double>::value ? 64 : 256;
     const size_t shm = sizeof(typename C2<R>::T) * (size_t)na * CJ;
     for (int j0 = 0; j0 < nb; j0 += CJ) {
@@ -842,14 +857,14 @@ template <typename R, int NB>
 void small_space_group(const void* V, int na, const double* d_signs, const void* X, int j0, int nj, void* Xp, void* Ys,
                        long long n, double2* d_C, double2* d_partial, long long partial_cap, cudaStream_t s) {
     typedef typename C2<R>::T T;
-    const int rowblocks = (na + 63) / 64;
+    const int rowblocks = (na + 63) / 64;  // (the chunks' lengths do not depend on the rows of a warp)
     long long nchunk = std::max(1LL, (4LL * 152) / rowblocks);
     const long long cap = partial_cap / ((long long)na * nj);
     if (nchunk > cap) nchunk = std::max(1LL, cap);
     long long chunk = (n + nchunk - 1) / nchunk;
     chunk = ((chunk + 31) / 32) * 32;
     nchunk = (n + chunk - 1) / chunk;
-    dim3 grid((unsigned)nchunk, rowblocks);
+    dim3 grid((unsigned)nchunk, sp_row_blocks(na, NB));
     vdot_rows_k<R, NB><<<grid, 256, 0, s>>>((const T*)V, n, na, (const T*)X + (long long)j0 * n, n, nj, n, chunk,
                                             d_partial);
     count_launch();
