@@ -266,11 +266,13 @@ __device__ __forceinline__ void add_exact(float& s, float& c, float x) {
     c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z)));
     s = t;
 }
-__device__ __forceinline__ void add_exact(double& s, double&, double x) { s += x; }
 
 // partial[r][b] = sum over this block's slice of conj(a) b (rhs r).  The sums of threads meet in FP64, whose
-// pipe bounds the block sums (1300 cycles a block): red_blocks() gives each thread at least eight elements, and
-// what FP32 would lose over them is kept.  12 vectors of 8^3 x 16, FP32: 49 -> 8.7 us (norms 29 -> 5.8 us) against
+// pipe bounds the block sums (1300 cycles a block): red_blocks() gives each thread at least eight elements.  What
+// FP32 would lose over them is kept, and a thread whose FP32 sum leaves FP32's range (eight numbers of 1e19 squared
+// do, one does not) adds its products in FP64.  FP64 adds them to two sums by turns: eight elements add a rounding
+// variance of 26 of their mean squares, 24 in the tree that blocks of one element a thread made of them, 35 in one
+// chain (four sums: 24, but 39 -> 50 us on 12 vectors of 8^3 x 16).  12 vectors of 8^3 x 16, FP32: 49 -> 8.7 us (norms 29 -> 5.8 us) against
 // 608 blocks a vector, which left a thread less than one element.
 template <typename R, bool NORM>
 __global__ void __launch_bounds__(RT) dot_partial_k(const typename C2<R>::T* __restrict__ a,
@@ -279,17 +281,44 @@ __global__ void __launch_bounds__(RT) dot_partial_k(const typename C2<R>::T* __r
     const int r = blockIdx.y;
     const typename C2<R>::T* pa = a + (long long)r * n;
     const typename C2<R>::T* pb = NORM ? pa : b + (long long)r * n;
-    R sre = 0, sim = 0, cre = 0, cim = 0;
-#pragma unroll 4
-    for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < n; i += (long long)gridDim.x * RT) {
+    const long long first = (long long)blockIdx.x * RT + threadIdx.x, step = (long long)gridDim.x * RT;
+    auto product = [&](long long i, R& re, R& im) {
         const typename C2<R>::T x = pa[i], y = NORM ? x : pb[i];
-        add_exact(sre, cre, fmad(x.y, y.y, x.x * y.x));
-        if (!NORM) add_exact(sim, cim, fmad(-x.y, y.x, x.x * y.y));
+        re = fmad(x.y, y.y, x.x * y.x);
+        im = NORM ? R(0) : fmad(-x.y, y.x, x.x * y.y);
+    };
+    double2 sum = make_double2(0, 0);
+    R re, im;
+    if constexpr (std::is_same<R, double>::value) {
+        double s[2] = {0, 0}, t[2] = {0, 0};
+        int q = 0;
+#pragma unroll 4
+        for (long long i = first; i < n; i += step) {
+            product(i, re, im);
+            s[q] += re;
+            if (!NORM) t[q] += im;
+            q ^= 1;
+        }
+        sum = make_double2(s[0] + s[1], t[0] + t[1]);
+    } else {
+        float sre = 0, sim = 0, cre = 0, cim = 0;
+#pragma unroll 4
+        for (long long i = first; i < n; i += step) {
+            product(i, re, im);
+            add_exact(sre, cre, re);
+            if (!NORM) add_exact(sim, cim, im);
+        }
+        if (isfinite(sre) && isfinite(sim)) {
+            sum = make_double2((double)sre + (double)cre, (double)sim + (double)cim);
+        } else {
+            for (long long i = first; i < n; i += step) {
+                product(i, re, im);
+                sum = dadd(sum, make_double2((double)re, (double)im));
+            }
+        }
     }
-    if (!isfinite(sre)) cre = 0;  // an overflowed sum stays what it is
-    if (!isfinite(sim)) cim = 0;
-    double2 tot = block_sum<RT>(make_double2((double)sre + (double)cre, (double)sim + (double)cim));
-    if (threadIdx.x == 0) partial[(long long)r * gridDim.x + blockIdx.x] = tot;
+    sum = block_sum<RT>(sum);
+    if (threadIdx.x == 0) partial[(long long)r * gridDim.x + blockIdx.x] = sum;
 }
 
 // out[r] = sum_b partial[r][b], fixed order
