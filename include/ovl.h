@@ -72,9 +72,13 @@ enum {
 
 enum { OV_BC_PERIODIC = 0, OV_BC_ANTIPERIODIC = 1, OV_BC_DIRICHLET = 2 };
 
-/* Arithmetic of operator applications. F64: FP64 storage and arithmetic; the polynomial recurrences run on
- * vectors of 57-bit integers with one exponent per site (every number to 2^-56 of the largest of its site;
- * a NaN or an infinity makes the whole site NaN), which is closer to the exact result than FP64 arithmetic.
+/* Arithmetic of operator applications. F64: FP64 storage and arithmetic.  The polynomial recurrences of the
+ * sign function, of its field derivative and of the eigensolver's filter run on vectors of 57-bit integers with
+ * one exponent per site where the links are of like size (rows and columns within a factor 4) and mix the colours
+ * at every site: every number is kept to 2^-56 of the largest of its site, which bounds the error of a site's vector
+ * below that of FP64 arithmetic, not that of a component far below the others (a NaN or an infinity makes the whole
+ * site NaN).  On other links (free, Abelian or nearly so, of very different sizes, not finite), and for the
+ * per-mode polynomials of a small space's derivative, the recurrences are in FP64.
  * F32: FP32 storage and arithmetic (reductions accumulate in FP64).
  * F16, BF16: the gauge links and the vectors of the Chebyshev recurrence are stored in 16
  * bits (FP16 with one FP32 scale per site, or BF16) and computed in FP32; the small-space

@@ -103,6 +103,7 @@ struct ov_ctx {
     void* U16 = nullptr;  // 16-bit links of an FP16 / BF16 context
     void* Ufx = nullptr;  // fixed-point links of the FP64 recurrences (made from U64 on first use)
     double fx_scale2 = 0.0;  // squared scale of the operator Ufx holds (0: none yet)
+    int fx_fit = -1;         // whether the links are ones for fixed point (-1: not looked at yet)
     bool gauge_set = false;
     std::vector<Bank> banks;
     std::vector<DefSpace> dspaces;  // D_ov deflation spaces per (phase, chirality)
@@ -189,7 +190,7 @@ size_t vec_bytes(const ov_ctx* c, int prec) {
     if (prec == OV_PREC_BF16) return (size_t)half_rhs_bytes<B16>(c->g.V);
     return (size_t)12 * c->g.V * (prec == OV_PREC_F64 ? 16 : 8);
 }
-double site_spinor_bytes(int prec) { return prec == OV_PREC_F64 ? 196 : prec == OV_PREC_F32 ? 96 : prec == OV_PREC_F16 ? 52 : 48; }
+double site_spinor_bytes(int prec) { return prec == OV_PREC_F64 ? 192 : prec == OV_PREC_F32 ? 96 : prec == OV_PREC_F16 ? 52 : 48; }
 // (16 bits: of two rows, which a link cannot do without; the third is stored for its instructions)
 double site_link_bytes(int prec) { return prec == OV_PREC_F64 ? 576 : prec == OV_PREC_F32 ? 192 : 96; }
 
@@ -412,6 +413,33 @@ bool any_phase(const SysSet& S) {
     return false;
 }
 
+// Whether the FP64 recurrences may run in fixed point on the present links (looked at once a gauge field).
+//
+// A fixed-point vector keeps a site's numbers to 2^-56 of the largest of them, links to 2^-56 of the largest of the
+// lattice, where FP64 keeps each number to 2^-53 of itself.  That is as good where what a number meets in the
+// next application is of the size of the largest around it: where every link has the size of the others
+// (rows and columns within a factor 4) and at every site each colour gets a fair share of each other colour, at least
+// 1/4 of the largest row over the site's eight hops (random links exp(i 0.2 H) get 1.7, with a smallest of 0.4 on
+// 65536 sites; exp(i 0.1 H) 0.9 and 0.2).  FP64 then rounds each component of H_w v by about 2^-53 1/4 of the
+// largest neighbour, and the fixed-point stencil by as much (eight hops rounded to 2^-56 of it).  Spins need no
+// test: two applications bring each spin to each other with coefficients of order 1.  Fields that do not mix colours so
+// (free, Abelian, nearly so), links of very different sizes and links that are not finite keep the FP64 stencil, five
+// times slower and exact to the last component.
+int fx_usable(ov_ctx* c, bool* ok, cudaStream_t s) {
+    if (c->fx_fit < 0) {
+        TRY(ensure_small(c, 0, 0, 64));
+        double v[3];
+        launch_fx_survey(c->g, c->U64, c->d_red, s);
+        CKL();
+        CK(cudaMemcpyAsync(v, c->d_red, sizeof(v), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        // (comparisons with a NaN are false)
+        c->fx_fit = std::isfinite(v[0]) && v[0] > 0.0 && v[1] >= v[0] / 16.0 && v[2] >= 0.25 * std::sqrt(v[0]);
+    }
+    *ok = c->fx_fit == 1;
+    return OV_OK;
+}
+
 // Links of the FP64 recurrences over the systems of S: the context's fixed-point links of
 // sqrt(scale2) H_w (made from the FP64 links when the scale changes), and for each distinct non-zero
 // phase the x links with that phase.
@@ -583,7 +611,6 @@ template <typename R, typename ST = R>
 int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogue fin, void* out, cudaStream_t s,
                   int degree = 0) {
     constexpr bool HALF = !std::is_same<R, ST>::value;
-    constexpr bool FX = std::is_same<ST, double>::value;  // the recurrence on fixed-point vectors
     const int prec = prec_of<R>();
     const int precs = prec_of<ST>();
     const int V = c->g.V;
@@ -592,13 +619,15 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
     TRY(upload_sys(c, S, s));
     const double* d_phase = any_phase(S) ? c->d_phase : nullptr;
 
+    bool fx = false;  // FP64: the recurrence on fixed-point vectors
+    if (std::is_same<ST, double>::value) TRY(fx_usable(c, &fx, s));
     void *xg, *xperp, *ys, *t, *bA, *bB;
     TRY(workspace(c, "sp_xg", prec, ns, &xg));
     TRY(workspace(c, "sp_xperp", prec, ns, &xperp));
     TRY(workspace(c, "sp_ys", prec, ns, &ys));
     void *xs = xperp, *p32 = nullptr;  // x_perp in the recurrence's storage; FP32 copy of its result
     FxLinks fxl;
-    if (FX) {
+    if (fx) {
         TRY(workspace_fx(c, "sp_t", ns, &t));
         TRY(workspace_fx(c, "sp_bA", ns, &bA));
         TRY(workspace_fx(c, "sp_bB", ns, &bB));
@@ -656,21 +685,21 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
     const double m0 = c->p.m0;
     const void* U = links_of<R>(c);
     const void* Us = links_of<ST>(c);
-    if (FX) TRY(fx_links(c, S, alpha, &fxl, s));
+    if (fx) TRY(fx_links(c, S, alpha, &fxl, s));
     // algorithmic bytes per site of one launch: links once (shared by the systems) plus each
     // system's input, output and epilogue vectors
-    const double Vd = (double)V, lb = site_link_bytes(precs), sb = site_spinor_bytes(precs);
+    const double Vd = (double)V, lb = site_link_bytes(precs), sb = fx ? 196 : site_spinor_bytes(precs);
     // the whole recurrence (2n launches, no host work) as one stream sequence
     // timing launches read t, bA, x_perp and write bB only (rewritten by the recurrence below)
-    const int nconv = FX ? 3 : (HALF ? 2 : 1);  // launches besides the recurrence
+    const int nconv = fx ? 3 : (HALF ? 2 : 1);  // launches besides the recurrence
     // half: the step's operator is (alpha / 2) H_w^2, which the links of the fixed-point recurrence do not carry
     auto step = [&](const void* in, void* o, const Epilogue& e, cudaStream_t st, int shape, bool half = false) {
-        if constexpr (FX) launch_fx_dslash(c->g, fxl, in, o, nullptr, ns, fx_epilogue(e, half), st, shape);
+        if (fx) launch_fx_dslash(c->g, fxl, in, o, nullptr, ns, fx_epilogue(e, half), st, shape);
         else launch_dslash<ST>(c->g, m0, Us, in, o, ns, d_phase, e, st, false, shape);
     };
     const int rb = tuned_shape<ST>(c, ns, t, bA, xs, bA, bB, s, step);
     auto enqueue = [&](cudaStream_t st) -> void* {
-        if constexpr (FX) {
+        if (fx) {
             launch_fx_from_f64(xperp, xs, V, ns, 1.0, st);
             launch_fx_from_f64(xperp, bA, V, ns, cf[n], st);
         } else if constexpr (HALF) {
@@ -698,7 +727,7 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
             b2 = b1;
             b1 = o;
         }
-        if constexpr (FX) {  // x_perp is not needed any more: its buffer takes P(Q^2) x_perp
+        if (fx) {  // x_perp is not needed any more: its buffer takes P(Q^2) x_perp
             launch_fx_to_f64(b1, xperp, V, ns, 1.0, st);
             b1 = xperp;
         }
@@ -719,7 +748,7 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
     if (c->use_graphs) {
         char key[384];
         snprintf(key, sizeof(key), "%d/%d/%d/%d/%p/%p/%p/%p/%p/%p/%p/%p/%p", precs, n, ns, rb, xperp, xs, bA, bB, t,
-                 (const void*)d_phase, FX ? fxl.links : Us, fxl.xlinks, (const void*)fxl.xidx);
+                 (const void*)d_phase, fx ? fxl.links : Us, fxl.xlinks, (const void*)fxl.xidx);
         auto it = c->graphs.find(key);
         if (it == c->graphs.end()) {
             if (!c->cap_stream) CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
@@ -971,27 +1000,27 @@ int register_bank_internal(ov_ctx* c, double phase, const void* W64, int n, cons
 }
 
 // Columns of the eigensolver's block per chunk of its filter and residual passes: three vectors of
-// precision prec per column within the context's budget, at least one column.
-int eig_chunk(const ov_ctx* c, int prec, int m) {
-    const size_t vb = prec == OV_PREC_F64 ? fx_rhs_bytes(c->g.V) : vec_bytes(c, prec);
-    const long long per_column = 3LL * (long long)vb;
+// precision prec (fx: fixed point) per column within the context's budget, at least one column.
+int eig_chunk(const ov_ctx* c, int prec, int m, bool fx = false) {
+    const long long per_column = 3LL * (long long)(fx ? fx_rhs_bytes(c->g.V) : vec_bytes(c, prec));
     return (int)std::max(1LL, std::min<long long>(m, c->eig_chunk_bytes / per_column));
 }
 
 // Chebyshev filter W <- T_d(Z) W (then normalised by the caller), Z = (2 Q^2 - (1 + a))/(1 - a),
 // which damps the part of the spectrum of Q^2 in [a, 1] and amplifies [0, a).  W: m vectors of
 // precision R, filtered a chunk of columns at a time (the recurrence acts on each column alone;
-// its three temporaries are chunk-sized).  FP64: the recurrence runs on fixed-point vectors.
+// its three temporaries are chunk-sized).  FP64: on fixed-point vectors where the links allow it.
 template <typename R>
 int cheb_filter(ov_ctx* c, void* W, int m, double a, int degree, const SysSet& S, const double* d_phase,
                 cudaStream_t s) {
-    constexpr bool FX = std::is_same<R, double>::value;
     const int prec = prec_of<R>();
     const size_t vb = vec_bytes(c, prec);
-    const int cw = eig_chunk(c, prec, m);
+    bool fx = false;
+    if (std::is_same<R, double>::value) TRY(fx_usable(c, &fx, s));
+    const int cw = eig_chunk(c, prec, m, fx);
     void *Tm, *Tc, *tt;
     FxLinks fxl;
-    if constexpr (FX) {
+    if (fx) {
         TRY(workspace_fx(c, "flt_Tm", cw, &Tm));
         TRY(workspace_fx(c, "flt_Tc", cw, &Tc));
         TRY(workspace_fx(c, "flt_t", cw, &tt));
@@ -1002,15 +1031,16 @@ int cheb_filter(ov_ctx* c, void* W, int m, double a, int degree, const SysSet& S
     }
     const double h = c->hw_norm, m0 = c->p.m0;
     const double za = 2.0 / ((1.0 - a) * h * h), zb = -(1.0 + a) / (1.0 - a);
-    if (FX) TRY(fx_links(c, S, 2.0 * za, &fxl, s));
+    const void* U = std::is_same<R, double>::value ? c->U64 : c->U32;
+    if (fx) TRY(fx_links(c, S, 2.0 * za, &fxl, s));
     for (int j0 = 0; j0 < m; j0 += cw) {
         const int nj = std::min(cw, m - j0);
         auto step = [&](const void* in, void* out, const Epilogue& e, bool half = false) {
-            if constexpr (FX) launch_fx_dslash(c->g, fxl, in, out, nullptr, nj, fx_epilogue(e, half), s, 0);
-            else launch_dslash<R>(c->g, m0, c->U32, in, out, nj, d_phase, e, s);
+            if (fx) launch_fx_dslash(c->g, fxl, in, out, nullptr, nj, fx_epilogue(e, half), s, 0);
+            else launch_dslash<R>(c->g, m0, U, in, out, nj, d_phase, e, s);
         };
         void* Wj = (char*)W + vb * j0;
-        if constexpr (FX) launch_fx_from_f64(Wj, Tm, c->g.V, nj, 1.0, s);  // T_0
+        if (fx) launch_fx_from_f64(Wj, Tm, c->g.V, nj, 1.0, s);  // T_0
         else CK(cudaMemcpyAsync(Tm, Wj, vb * nj, cudaMemcpyDeviceToDevice, s));
         Epilogue plain;
         step(Tm, tt, plain);
@@ -1032,9 +1062,9 @@ int cheb_filter(ov_ctx* c, void* W, int m, double a, int degree, const SysSet& S
             step(tt, tkm, e);  // T_{k+1} written over T_{k-1}
             std::swap(tk, tkm);
         }
-        if constexpr (FX) launch_fx_to_f64(tk, Wj, c->g.V, nj, 1.0, s);
+        if (fx) launch_fx_to_f64(tk, Wj, c->g.V, nj, 1.0, s);
         CKL();
-        if constexpr (!FX) CK(cudaMemcpyAsync(Wj, tk, vb * nj, cudaMemcpyDeviceToDevice, s));
+        if (!fx) CK(cudaMemcpyAsync(Wj, tk, vb * nj, cudaMemcpyDeviceToDevice, s));
     }
     c->dslash_count += 2LL * degree * m;
     return OV_OK;
@@ -1313,6 +1343,7 @@ int ov_set_gauge(ov_ctx* c, const void* U, int dtype, ov_stream_t stream) {
     }
     launch_pack_gauge<double>(U, dtype, c->U64, c->g, s);
     c->fx_scale2 = 0.0;
+    c->fx_fit = -1;
     launch_pack_gauge<float>(U, dtype, c->U32, c->g, s);
     if (c->p.precision == OV_PREC_F16) launch_pack_gauge_half<H16>(U, dtype, c->U16, c->g.V, s);
     if (c->p.precision == OV_PREC_BF16) launch_pack_gauge_half<B16>(U, dtype, c->U16, c->g.V, s);
@@ -2984,7 +3015,84 @@ int prepare_bank_derivative(ov_ctx* c, Bank* b, cudaStream_t s) {
 // of the Clenshaw recurrence b_k = c_k x + 2 Y b_{k+1} - b_{k+2} with x fixed:
 //   db_k = 2 dY b_{k+1} + 2 Y db_{k+1} - db_{k+2},  2 dY = alpha (dH H + H dH),
 // and d(Q p) = (dH p + H dp)/h.
+int tangent_poly_f64(ov_ctx* c, const void* X, const SysSet& S, void* Y, cudaStream_t s) {
+    const int ns = S.n;
+    const long long n12 = 12LL * c->g.V;
+    const size_t vb = vec_bytes(c, OV_PREC_F64);
+    void *bA, *bB, *dA, *dB, *t, *u, *sv, *r;
+    TRY(workspace(c, "tg_bA", OV_PREC_F64, ns, &bA));
+    TRY(workspace(c, "tg_bB", OV_PREC_F64, ns, &bB));
+    TRY(workspace(c, "tg_dA", OV_PREC_F64, ns, &dA));
+    TRY(workspace(c, "tg_dB", OV_PREC_F64, ns, &dB));
+    TRY(workspace(c, "tg_t", OV_PREC_F64, ns, &t));
+    TRY(workspace(c, "tg_u", OV_PREC_F64, ns, &u));
+    TRY(workspace(c, "tg_s", OV_PREC_F64, ns, &sv));
+    TRY(workspace(c, "tg_r", OV_PREC_F64, ns, &r));
+    TRY(upload_sys(c, S, s));
+    const double* d_phase = any_phase(S) ? c->d_phase : nullptr;
+    const int n = c->p.poly_degree;
+    const double eps = c->p.eps, h = c->hw_norm, m0 = c->p.m0;
+    const double alpha = 4.0 / ((1.0 - eps) * h * h);
+    const double beta = -2.0 * (1.0 + eps) / (1.0 - eps);
+    const void* U = c->U64;
+    launch_scale<double>(c->coeffs[n], X, bA, ns * n12, s);
+    CK(cudaMemsetAsync(dA, 0, vb * ns, s));
+    void *b1 = bA, *b2 = nullptr, *db1 = dA, *db2 = nullptr;
+    Epilogue plain, derv;
+    for (int k = n - 1; k >= 0; --k) {
+        const double hf = (k == 0) ? 0.5 : 1.0;
+        launch_dslash<double>(c->g, m0, U, b1, t, ns, d_phase, plain, s);          // t = H b1
+        launch_dslash<double>(c->g, m0, U, b1, u, ns, d_phase, derv, s, true);     // u = dH b1
+        Epilogue es;
+        es.c1 = 1.0;
+        es.v1 = u;
+        launch_dslash<double>(c->g, m0, U, db1, sv, ns, d_phase, es, s);           // s = H db1 + u
+        launch_dslash<double>(c->g, m0, U, t, r, ns, d_phase, derv, s, true);      // r = dH t
+        Epilogue eb;
+        eb.c_op = alpha * hf;
+        eb.c1 = beta * hf;
+        eb.v1 = b1;
+        eb.c2 = c->coeffs[k];
+        eb.v2 = X;
+        eb.c3 = -1.0;
+        eb.v3 = b2;
+        void* ob = b2 ? b2 : bB;
+        launch_dslash<double>(c->g, m0, U, t, ob, ns, d_phase, eb, s);             // b_k
+        Epilogue ed;
+        ed.c_op = alpha * hf;
+        ed.c1 = beta * hf;
+        ed.v1 = db1;
+        ed.c2 = alpha * hf;
+        ed.v2 = r;
+        ed.c3 = -1.0;
+        ed.v3 = db2;
+        void* od = db2 ? db2 : dB;
+        launch_dslash<double>(c->g, m0, U, sv, od, ns, d_phase, ed, s);            // db_k
+        b2 = b1;
+        b1 = ob;
+        db2 = db1;
+        db1 = od;
+    }
+    CKL();
+    c->dslash_count += 6LL * n * ns;
+    // Y = (H dp + dH p)/h with p = b1, dp = db1
+    Epilogue ep;
+    ep.c_op = 1.0 / h;
+    launch_dslash<double>(c->g, m0, U, b1, t, ns, d_phase, ep, s, true);           // t = dH p / h
+    Epilogue ey;
+    ey.c_op = 1.0 / h;
+    ey.c1 = 1.0;
+    ey.v1 = t;
+    launch_dslash<double>(c->g, m0, U, db1, Y, ns, d_phase, ey, s);
+    CKL();
+    return OV_OK;
+}
+
+// The same on fixed-point vectors where the links allow it.
 int tangent_poly(ov_ctx* c, const void* X, const SysSet& S, void* Y, cudaStream_t s) {
+    bool fx = false;
+    TRY(fx_usable(c, &fx, s));
+    if (!fx) return tangent_poly_f64(c, X, S, Y, s);
     const int ns = S.n;
     void *x, *bA, *bB, *dA, *dB, *t, *u, *sv;
     TRY(workspace_fx(c, "tg_x", ns, &x));

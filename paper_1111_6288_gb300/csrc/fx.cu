@@ -1,4 +1,5 @@
-// The recurrences of the FP64 operators on the integer pipes (fx_arith.h, fx_site.h).
+// The recurrences of the FP64 operators on the integer pipes (fx_arith.h, fx_site.h), on links that launch_fx_survey
+// finds fit for it.
 //
 // Every step of the polynomial Q P(Q^2) (Sec. 2) in FP64 is one application of H_w.  The FP64 stencil
 // (dslash_kernel<double>) keeps this GPU's FP64 pipe 91 % busy at 2 multiply-adds per clock and SM, so
@@ -361,6 +362,60 @@ __global__ void fx_link_norm_k(const double2* __restrict__ U, int V, unsigned lo
     if ((threadIdx.x & 31) == 0) atomicMax(out, best);
 }
 
+// Smallest of the warp's values, given as bits of doubles that are not negative.
+__device__ __forceinline__ unsigned long long warp_min(unsigned long long v) {
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long w = __shfl_down_sync(0xffffffffu, v, o);
+        v = w < v ? w : v;
+    }
+    return v;
+}
+
+// out[1], out[2] of launch_fx_survey (out[0] is fx_link_norm_k's): a thread per site, the links of its eight hops
+__global__ void __launch_bounds__(128) fx_survey_k(const double2* __restrict__ U, Geom g, unsigned long long* __restrict__ out) {
+    unsigned long long least = ~0ULL, mixed = ~0ULL;
+    const int V = g.V;
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < V; s += gridDim.x * blockDim.x) {
+        double share[3][3] = {};
+        double norm = INFINITY;
+        int rest = s, stride = 1;
+        for (int mu = 0; mu < 4; ++mu) {
+            const int L = g.L[mu], x = rest % L;
+            rest /= L;
+            const bool open = g.bcf[mu] == 0.0;
+            for (int back = 0; back < 2; ++back) {
+                if (open && x == (back ? 0 : L - 1)) continue;
+                const int site = back ? (x == 0 ? s + (L - 1) * stride : s - stride) : s;
+                const double2* u = U + (i64)mu * 9 * V + site;
+                double row[3] = {0, 0, 0}, col[3] = {0, 0, 0};
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    const double2 z = u[(i64)k * V];
+                    const double q = z.x * z.x + z.y * z.y, m = fmax(fabs(z.x), fabs(z.y));
+                    row[k / 3] += q;
+                    col[k % 3] += q;
+                    // forward: entry (a, b) brings b to a; backward, U^+: b = row, a = column
+                    if (back) share[k % 3][k / 3] += m;
+                    else share[k / 3][k % 3] += m;
+                }
+#pragma unroll
+                for (int i = 0; i < 3; ++i) norm = fmin(norm, fmin(row[i], col[i]));
+            }
+            stride *= L;
+        }
+        const double a = fmin(fmin(share[0][1], share[1][0]), fmin(share[0][2], share[2][0]));
+        const double m = fmin(a, fmin(share[1][2], share[2][1]));
+        least = min(least, (unsigned long long)__double_as_longlong(norm));
+        mixed = min(mixed, (unsigned long long)__double_as_longlong(m));
+    }
+    least = warp_min(least);
+    mixed = warp_min(mixed);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMin(out + 1, least);
+        atomicMin(out + 2, mixed);
+    }
+}
+
 // a 2^k to the nearest integer, a = hi + lo
 __device__ __forceinline__ i64 to_int(double hi, double lo, int k) {
     return __double2ll_rn(scalbn(hi, k)) + __double2ll_rn(scalbn(lo, k));
@@ -536,6 +591,15 @@ void fx_launch(const fx::Args& a, dim3 grid, dim3 block, int nrhs, cudaStream_t 
     fx_dslash_kernel<EPI, DUAL><<<grid, block, smem, s>>>(a, nrhs);
 }
 }  // namespace
+
+void launch_fx_survey(const Geom& g, const void* U64, void* out, cudaStream_t s) {
+    unsigned long long* o = (unsigned long long*)out;
+    cudaMemsetAsync(o, 0, 8, s);
+    cudaMemsetAsync(o + 1, 0x7f, 16, s);  // 1e306, above every norm that counts
+    fx_link_norm_k<<<(int)std::min<i64>((4LL * g.V + 255) / 256, 152 * 8), 256, 0, s>>>((const double2*)U64, g.V, o);
+    fx_survey_k<<<std::min((g.V + 127) / 128, 152 * 8), 128, 0, s>>>((const double2*)U64, g, o);
+    count_launch(2);
+}
 
 void launch_fx_links(const Geom& g, double m0, double scale2, const void* U64, void* dst, cudaStream_t s) {
     fx::Scale* sc = scale_of(dst, g.V);

@@ -111,6 +111,10 @@ struct FxEpilogue {
 size_t fx_rhs_bytes(int V);
 size_t fx_link_bytes(int V);
 size_t fx_xlink_bytes(int V);
+// What the links are like: out[0..2] = the largest squared row or column norm of a link (a NaN: not finite), the
+// smallest of the links that hops use, and the smallest, over sites and pairs of colours a != b, of the sum over the
+// site's hops of max(|re|, |im|) of the entry that brings colour b to a.  U64: the FP64 stencil's links.
+void launch_fx_survey(const Geom& g, const void* U64, void* out, cudaStream_t s);
 // Links of g H_w, g = sqrt(scale2).
 void launch_fx_links(const Geom& g, double m0, double scale2, const void* U64, void* dst, cudaStream_t s);
 void launch_fx_xlinks(const Geom& g, double scale2, const void* U64, const void* links, void* dst,

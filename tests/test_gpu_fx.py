@@ -137,3 +137,120 @@ def test_operator_coefficients_that_are_powers_of_two(P, hw, eps, degree):
     growth = np.cosh(degree * np.arccosh(max(ends)))
     assert np.linalg.norm(y[0] - want) <= bound(degree) * growth * np.linalg.norm(x[0])
     assert np.linalg.norm(want) > 1e3 * bound(degree) * growth * np.linalg.norm(x[0])
+
+
+# ---- links that fixed point is not for: each number keeps FP64's own precision ----------------------
+
+
+def decoupled_links(kind, dims):
+    """Links that do not mix colour 2 with the others ("blocks"), or no colours at all."""
+    V = synth.volume(dims)
+    rng = np.random.default_rng(31)
+    U = np.zeros((4, V, 3, 3), complex)
+    if kind == "unit":
+        U[:] = np.eye(3)
+    elif kind == "diagonal":
+        U[..., range(3), range(3)] = np.exp(1j * rng.uniform(-np.pi, np.pi, (4, V, 3)))
+    else:
+        A = rng.standard_normal((4, V, 2, 2)) + 1j * rng.standard_normal((4, V, 2, 2))
+        U[..., :2, :2] = np.linalg.qr(A)[0]
+        U[..., 2, 2] = np.exp(1j * rng.uniform(-np.pi, np.pi, (4, V)))
+    return U.reshape((4,) + synth.site_shape(dims) + (3, 3))
+
+
+@pytest.mark.parametrize("op", ["sign", "overlap", "derivative"])
+@pytest.mark.parametrize("kind", ["unit", "diagonal", "blocks"])
+@pytest.mark.parametrize("dims", [(4, 3, 2, 5), (8, 8, 8, 16)])
+def test_colours_that_do_not_mix_keep_their_own_precision(P, dims, kind, op):
+    """Colour 2 at 1e-18 of the others gives what it gives alone, to the last bit: the others enter it only
+    through links that are zero."""
+    import torch
+
+    ctx = P.Context(P.Params(dims=dims, bc=(0, 0, 0, 1), m0=M0, eps=0.1, poly_degree=4, max_nrhs=2))
+    ctx.set_gauge(dev(decoupled_links(kind, dims)))
+    if op == "derivative":
+        P.deflate(ctx, None, [], phase=0.3)
+    x = np.repeat(synth.gaussian_spinor(dims, 1, 32), 2, axis=0)
+    x[..., 2] *= 1e-18
+    x[1, ..., :2] = 0.0
+    xd = dev(x)
+    y = torch.empty_like(xd)
+    if op == "sign":
+        P.apply_sign_Hw(ctx, xd, y)
+    elif op == "overlap":
+        P.apply_overlap(ctx, xd, y, mass=0.1)
+    else:
+        P.apply_dDdphi(ctx, xd, y, 0.1, phase=[0.3, 0.3])
+    ctx.close()
+    y = y.cpu().numpy()
+    assert np.abs(y[1, ..., 2]).max() > 0.0
+    assert np.array_equal(y[0, ..., 2], y[1, ..., 2])
+
+
+def test_links_of_very_different_sizes(P):
+    """Half of the lattice with links 2^-40 times the other's, m0 = -4 (no term without a link): the derivative
+    in that half, dH/dphi P(Q^2) x / h up to terms 2^-80 of it, is as accurate relative to its own size as with
+    equal links."""
+    import torch
+
+    from oracle import derivative
+
+    dims, bc, degree, hw, phase = (3, 4, 2, 14), (0, 0, 0, 2), 1, 4.0, 0.3
+    U = synth.random_su3_field(dims, 0.3, seed=33)
+    U[:, 7:] *= 2.0**-40
+    x = synth.gaussian_spinor(dims, 1, 34)
+    x[:, :11] = 0.0  # 2 n + 1 = 3 hops from the other half
+    ctx = P.Context(P.Params(dims=dims, bc=bc, m0=-4.0, hw_norm=hw, eps=0.02, poly_degree=degree, max_nrhs=1))
+    ctx.set_gauge(dev(U))
+    P.deflate(ctx, None, [], phase=phase)
+    xd = dev(x)
+    y = torch.empty_like(xd)
+    P.apply_dDdphi(ctx, xd, y, 0.0, phase=[phase])
+    ctx.close()
+    p = ov.OverlapParams(m0=-4.0, hw_norm=hw, eps=0.02, degree=degree, bc=(1.0, 1.0, 1.0, 0.0))
+    px = ov.apply_poly_Q2(U, x[0], p, phase)
+    want = derivative.dhw_dphi(U, px, p.bc, phase) / hw
+    want[..., 2:, :] *= -1  # gamma5
+    assert np.linalg.norm(want) > 0.0
+    assert np.linalg.norm(y.cpu().numpy()[0] - want) <= bound(degree) * np.linalg.norm(want)
+
+
+def test_a_nan_in_one_link(P):
+    """It reaches the sites within 2 n + 1 hops, zeros included, and no others; in a link that no hop uses it
+    reaches none."""
+    dims, bc, degree = (4, 4, 2, 14), (0, 0, 0, 2), 1
+    U = synth.random_su3_field(dims, 0.3, seed=35)
+    x = synth.gaussian_spinor(dims, 1, 36)
+    x[0, :3] = 0.0
+    bad = U.copy()
+    bad[0, 0, 0, 0, 0, 1, 1] = np.nan  # the x link of the first site
+    y, hw = run(P, dims, bc, bad, x, degree, [0.0])
+    want = oracle_sign(U, x[0], bc, hw, degree, 0.0)
+    assert np.isnan(y[0, 0, 0, 0, :2]).any()
+    assert np.linalg.norm(y[0, 4:] - want[4:]) <= bound(degree) * np.linalg.norm(want[4:])
+    bad = U.copy()
+    bad[3, -1] = np.nan  # the time links across the Dirichlet face
+    y, hw = run(P, dims, bc, bad, x, degree, [0.0])
+    assert np.linalg.norm(y[0] - want) <= bound(degree) * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("spread, fixed", [(0.2, True), (0.4, True), (0.02, False)])
+def test_which_fields_take_fixed_point(P, spread, fixed):
+    """The recurrence's bytes a site tell: 196 of a fixed-point vector, 192 of an FP64 one (two applications,
+    links of 576, seven vectors but for the first)."""
+    import torch
+
+    dims, degree = (6, 6, 6, 8), 4
+    U = synth.random_su3_field(dims, spread, seed=37)
+    x = synth.gaussian_spinor(dims, 1, 38)
+    ctx = P.Context(P.Params(dims=dims, bc=(0, 0, 0, 1), m0=M0, eps=0.02, poly_degree=degree, max_nrhs=1))
+    ctx.set_gauge(dev(U))
+    ctx.set_profiling(True)
+    xd = dev(x)
+    y = torch.empty_like(xd)
+    P.apply_sign_Hw(ctx, xd, y)
+    want = oracle_sign(U, x[0], (0, 0, 0, 1), ctx.hw_norm, degree, 0.0)
+    vectors = 7 * degree - 1
+    assert ctx.read_profile(0)["clenshaw_bytes"] == synth.volume(dims) * (2 * degree * 576 + vectors * (196 if fixed else 192))
+    ctx.close()
+    assert np.linalg.norm(y.cpu().numpy()[0] - want) <= bound(degree) * np.linalg.norm(want)
