@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(FX_THREADS, kBlocksPerSm) fx_dslash_kernel(con
                 int4* o = fx::at(a.out2 + off, s);
                 fx::store_spin(o, f, fu);
                 fx::store_spin(o, 3 - f, fl);
-                if (f == 0) *fx::exponent_at(a.out2 + off, s) = H.bad ? fx::kNanExp : ed;
+                if (f == 0) *fx::exponent_at(a.out2 + off, s) = fx::bad_x(H) ? fx::kNanExp : ed;
             }
         }
     }
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(128) fx_split_kernel(const __grid_constant__ f
                 int4* o = fx::at(a.out2 + off, s);
                 fx::store_spin(o, f, fu);
                 fx::store_spin(o, 3 - f, fl);
-                if (f == 0) *fx::exponent_at(a.out2 + off, s) = H.bad ? fx::kNanExp : ed;
+                if (f == 0) *fx::exponent_at(a.out2 + off, s) = fx::bad_x(H) ? fx::kNanExp : ed;
             }
         }
         const i64 neg = k == 0 ? -(i64)f : 0;  // the y hops' lower spin; the z hops' has its sign already
@@ -487,7 +487,7 @@ __global__ void fx_xlinks_k(const double2* __restrict__ U, char* __restrict__ ou
     }
 }
 
-// FP64 spinors (12 planes of double2) times factor -> fixed point
+// FP64 spinors (12 planes of double2) times factor -> fixed point (factor 0: zeros, whatever they are)
 __global__ void __launch_bounds__(128) fx_from_f64_k(const double2* __restrict__ in, char* __restrict__ out, int V,
                                                      double factor) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -498,8 +498,8 @@ __global__ void __launch_bounds__(128) fx_from_f64_k(const double2* __restrict__
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
         p[k] = q[(i64)k * V];
-        p[k].x *= factor;
-        p[k].y *= factor;
+        p[k].x = factor == 0.0 ? 0.0 : p[k].x * factor;
+        p[k].y = factor == 0.0 ? 0.0 : p[k].y * factor;
         const unsigned long long x = (unsigned long long)__double_as_longlong(p[k].x) & 0x7fffffffffffffffULL;
         const unsigned long long y = (unsigned long long)__double_as_longlong(p[k].y) & 0x7fffffffffffffffULL;
         top = x > top ? x : top;

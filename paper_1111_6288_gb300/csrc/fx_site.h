@@ -365,6 +365,9 @@ FX_FN void half_hop(Half& H, const int4* pa, const int4* pb, const int4* u, i64 
     }
 }
 
+// Whether an x hop brings a NaN (the derivative has no other hops).
+FX_FN bool bad_x(const Half& H) { return H.ex[6] > kNanTest || H.ex[7] > kNanTest; }
+
 // The x hops of DUAL: F + B into the sums, F - B (spins f and 3 - f) left in fu, fl; returns its exponent.
 FX_FN int dual_split(Half& H, i64 (&fu)[6], i64 (&fl)[6], const i64 (&bu)[6], const i64 (&bl)[6]) {
     const int xref = H.ex[6] > H.ex[7] ? H.ex[6] : H.ex[7];

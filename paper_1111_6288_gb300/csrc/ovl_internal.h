@@ -119,7 +119,7 @@ void launch_fx_survey(const Geom& g, const void* U64, void* out, cudaStream_t s)
 void launch_fx_links(const Geom& g, double m0, double scale2, const void* U64, void* dst, cudaStream_t s);
 void launch_fx_xlinks(const Geom& g, double scale2, const void* U64, const void* links, void* dst,
                       const double* d_phases, int nphase, cudaStream_t s);
-// FP64 spinors (internal layout) times factor -> fixed point, and back (times factor).
+// FP64 spinors (internal layout) times factor -> fixed point (0: zeros, whatever they are), and back (times factor).
 void launch_fx_from_f64(const void* in, void* out, int V, int nrhs, double factor, cudaStream_t s);
 void launch_fx_to_f64(const void* in, void* out, int V, int nrhs, double factor, cudaStream_t s);
 // One application on fixed-point vectors.  out_deriv (may be null): g dH_w/dphi in, without the

@@ -254,3 +254,27 @@ def test_which_fields_take_fixed_point(P, spread, fixed):
     assert ctx.read_profile(0)["clenshaw_bytes"] == synth.volume(dims) * (2 * degree * 576 + vectors * (196 if fixed else 192))
     ctx.close()
     assert np.linalg.norm(y.cpu().numpy()[0] - want) <= bound(degree) * np.linalg.norm(want)
+
+
+def test_a_nan_reaches_the_derivative_through_x_hops_only(P):
+    """dH/dphi has x hops only, and the derivative's recurrence starts from zeros: three y hops from a NaN, the
+    result of degree 1 is what it is without."""
+    import torch
+
+    dims = (6, 8, 2, 4)
+    U = synth.random_su3_field(dims, 0.3, seed=39)
+    x = synth.gaussian_spinor(dims, 1, 40)
+    ctx = P.Context(P.Params(dims=dims, bc=(0, 0, 0, 1), m0=M0, eps=0.02, poly_degree=1, max_nrhs=1))
+    ctx.set_gauge(dev(U))
+    P.deflate(ctx, None, [], phase=0.3)
+    y = []
+    for value in (x[0, 1, 0, 0, 2, 0, 0], np.nan):
+        x[0, 1, 0, 0, 2, 0, 0] = value
+        xd = dev(x)
+        yd = torch.empty_like(xd)
+        P.apply_dDdphi(ctx, xd, yd, 0.0, phase=[0.3])
+        y.append(yd.cpu().numpy())
+    ctx.close()
+    assert np.isnan(y[1][0, 1, 0, 1, 1]).all() and not np.isnan(y[0]).any()
+    for far in (3, 5):
+        assert np.array_equal(y[1][0, 1, 0, far, 2], y[0][0, 1, 0, far, 2])
