@@ -126,7 +126,7 @@ struct ov_ctx {
     // optional CUDA-event timing of the Clenshaw loops (the Wilson kernels of the polynomial)
     // CUDA graphs of the Clenshaw loop, keyed by precision, systems and buffers
     bool use_graphs = true;
-    // autotuned right-hand sides per Wilson-kernel block, keyed by precision and systems
+    // autotuned right-hand sides per Wilson-kernel block, keyed by precision (or kTuneFx) and systems
     std::map<std::pair<int, int>, int> launch_shape;
     // small-space projection of 8 or more FP32 vectors: 1 = CUDA cores, 0 and 2 = tensor cores; the
     // (bank size, batch) pairs in the tuning log
@@ -491,20 +491,24 @@ FxEpilogue fx_epilogue(const Epilogue& e, bool half) {
     return f;
 }
 
+constexpr int kTuneFx = 4;  // beside the precisions in the key of a tuned shape
+
 // Launch shape of the Wilson kernel for ns systems of storage type R (right-hand sides per block;
 // for FP32 arithmetic also the 6- or 7-blocks-per-SM register budget and, where the lattice
 // allows, the tiled kernel): timed once on the sign pipeline's own buffers (the Clenshaw-step
 // launch with its epilogue), fastest kept.
-// launch(in, out, epilogue, stream, shape) enqueues one application.
+// launch(in, out, epilogue, stream, shape) enqueues one application.  fx: the fixed-point kernels, whose blocks
+// differ up to fx_block_rhs() right-hand sides only.
 template <typename R, typename F>
-int tuned_shape(ov_ctx* c, int ns, void* in, void* v1, void* v2, void* v3, void* out, cudaStream_t s, F launch) {
+int tuned_shape(ov_ctx* c, int ns, bool fx, void* in, void* v1, void* v2, void* v3, void* out, cudaStream_t s, F launch) {
     if (c->p.launch_shape > 0) return c->p.launch_shape;  // fixed by the caller
-    const auto key = std::make_pair(prec_of<R>(), ns);
+    const auto key = std::make_pair(fx ? kTuneFx : prec_of<R>(), ns);
+    const int most = std::min(ns, fx ? fx_block_rhs(c->g.V, ns) : 8);
     auto it = c->launch_shape.find(key);
     if (it != c->launch_shape.end()) return it->second;
     std::vector<int> shapes;
     for (int by : {1, 2, 4, 8}) {
-        if (by > ns) break;
+        if (by > most) break;
         shapes.push_back(by);
         if (!std::is_same<R, double>::value) {
             shapes.push_back(by | kShapeDense);
@@ -548,6 +552,8 @@ int tuned_shape(ov_ctx* c, int ns, void* in, void* v1, void* v2, void* v3, void*
         c->tune_log += "; ";
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
+    } else if (ns > 1) {
+        c->tune_log += std::to_string(ns) + " systems of few sites, one shape; ";
     }
     c->launch_shape[key] = best;
     return best;
@@ -697,7 +703,7 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
         if (fx) launch_fx_dslash(c->g, fxl, in, o, nullptr, ns, fx_epilogue(e, half), st, shape);
         else launch_dslash<ST>(c->g, m0, Us, in, o, ns, d_phase, e, st, false, shape);
     };
-    const int rb = tuned_shape<ST>(c, ns, t, bA, xs, bA, bB, s, step);
+    const int rb = tuned_shape<ST>(c, ns, fx, t, bA, xs, bA, bB, s, step);
     auto enqueue = [&](cudaStream_t st) -> void* {
         if (fx) {
             launch_fx_from_f64(xperp, xs, V, ns, 1.0, st);

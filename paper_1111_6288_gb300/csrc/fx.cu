@@ -634,6 +634,17 @@ void launch_fx_to_f64(const void* in, void* out, int V, int nrhs, double factor,
     count_launch();
 }
 
+namespace {
+bool fx_split(int V, int nrhs) { return (i64)((V + 15) / 16) * nrhs <= kSplitBlocks; }
+int fx_threads(int V, int nrhs) {
+    int threads = FX_THREADS;
+    while (threads > 32 && 2LL * V * nrhs < 152LL * 2 * threads) threads /= 2;
+    return threads;
+}
+}  // namespace
+
+int fx_block_rhs(int V, int nrhs) { return fx_split(V, nrhs) ? 1 : fx_threads(V, nrhs) / 32; }
+
 void launch_fx_dslash(const Geom& g, const FxLinks& U, const void* in, void* out, void* out_deriv, int nrhs,
                       const FxEpilogue& e, cudaStream_t s, int shape) {
     fx::Args a;
@@ -661,8 +672,7 @@ void launch_fx_dslash(const Geom& g, const FxLinks& U, const void* in, void* out
     for (int k = 0; k < 3; ++k) a.div[k] = fx::make_div((uint32_t)g.L[k]);
     a.V = g.V;
     const bool epi = e.v1 || e.v2 || e.v3 || e.half;
-    const i64 split_blocks = (i64)((g.V + 15) / 16) * nrhs;
-    if (split_blocks <= kSplitBlocks) {
+    if (fx_split(g.V, nrhs)) {
         const dim3 grid((g.V + 15) / 16, nrhs);
         if (out_deriv) {
             if (epi) fx_split_kernel<true, true><<<grid, 128, 0, s>>>(a);
@@ -674,10 +684,9 @@ void launch_fx_dslash(const Geom& g, const FxLinks& U, const void* in, void* out
         count_launch();
         return;
     }
-    int threads = FX_THREADS;
-    while (threads > 32 && 2LL * g.V * nrhs < 152LL * 2 * threads) threads /= 2;
+    const int threads = fx_threads(g.V, nrhs);
     int by = (shape & kShapeRhsMask) > 0 ? (shape & kShapeRhsMask) : 4;
-    by = std::min(by, threads / 32);
+    by = std::min(by, fx_block_rhs(g.V, nrhs));
     while (by > 1 && by > nrhs) by >>= 1;
     const int bx = threads / by, sites = bx / 2;
     const dim3 block(bx, by), grid((g.V + sites - 1) / sites, (nrhs + by - 1) / by);

@@ -122,6 +122,8 @@ void launch_fx_xlinks(const Geom& g, double scale2, const void* U64, const void*
 // FP64 spinors (internal layout) times factor -> fixed point (0: zeros, whatever they are), and back (times factor).
 void launch_fx_from_f64(const void* in, void* out, int V, int nrhs, double factor, cudaStream_t s);
 void launch_fx_to_f64(const void* in, void* out, int V, int nrhs, double factor, cudaStream_t s);
+// Most right-hand sides per block that a launch's shape makes a difference up to.
+int fx_block_rhs(int V, int nrhs);
 // One application on fixed-point vectors.  out_deriv (may be null): g dH_w/dphi in, without the
 // epilogue.  shape: right-hand sides per thread block in the low bits (0: default).
 void launch_fx_dslash(const Geom& g, const FxLinks& U, const void* in, void* out, void* out_deriv, int nrhs,

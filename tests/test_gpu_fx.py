@@ -278,3 +278,17 @@ def test_a_nan_reaches_the_derivative_through_x_hops_only(P):
     assert np.isnan(y[1][0, 1, 0, 1, 1]).all() and not np.isnan(y[0]).any()
     for far in (3, 5):
         assert np.array_equal(y[1][0, 1, 0, far, 2], y[0][0, 1, 0, far, 2])
+
+
+@pytest.mark.parametrize("dims, nrhs, shapes", [((4, 4, 4, 4), 8, []), ((8, 8, 8, 8), 8, [1, 2, 4]), ((8, 8, 8, 16), 3, [1, 2]),
+                                                ((8, 8, 8, 16), 1, [])])
+def test_only_shapes_that_differ_are_timed(P, dims, nrhs, shapes):
+    """Blocks of more than four systems do not exist, and eight lanes a site take no shape at all."""
+    import re
+
+    ctx = P.Context(P.Params(dims=dims, m0=M0, eps=0.02, poly_degree=2, max_nrhs=nrhs))
+    ctx.set_gauge(dev(synth.random_su3_field(dims, 0.3, seed=41)))
+    x = dev(synth.gaussian_spinor(dims, nrhs, 42))
+    P.apply_sign_Hw(ctx, x, x.clone())
+    assert [int(k) for k in re.findall(r"(\d+)d?t?:", ctx.tune_info)] == shapes
+    ctx.close()
