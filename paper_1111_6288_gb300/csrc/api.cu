@@ -21,6 +21,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <map>
 #include <numeric>
 #include <set>
@@ -104,6 +105,7 @@ struct ov_ctx {
     void* Ufx = nullptr;  // fixed-point links of the FP64 recurrences (made from U64 on first use)
     double fx_scale2 = 0.0;  // squared scale of the operator Ufx holds (0: none yet)
     int fx_fit = -1;         // whether the links are ones for fixed point (-1: not looked at yet)
+    long long fx_no_room = 0;  // fewest systems the device had no memory for in fixed point (0: none)
     bool gauge_set = false;
     std::vector<Bank> banks;
     std::vector<DefSpace> dspaces;  // D_ov deflation spaces per (phase, chirality)
@@ -413,7 +415,8 @@ bool any_phase(const SysSet& S) {
     return false;
 }
 
-// Whether the FP64 recurrences may run in fixed point on the present links (looked at once a gauge field).
+// Whether an FP64 recurrence over nvec systems may run in fixed point on the present links (looked at once a gauge
+// field).
 //
 // A fixed-point vector keeps a site's numbers to 2^-56 of the largest of them, links to 2^-56 of the largest of the
 // lattice, where FP64 keeps each number to 2^-53 of itself.  That is as good where what a number meets in the
@@ -425,7 +428,7 @@ bool any_phase(const SysSet& S) {
 // test: two applications bring each spin to each other with coefficients of order 1.  Fields that do not mix colours so
 // (free, Abelian, nearly so), links of very different sizes and links that are not finite keep the FP64 stencil, five
 // times slower and exact to the last component.
-int fx_usable(ov_ctx* c, bool* ok, cudaStream_t s) {
+int fx_usable(ov_ctx* c, long long nvec, bool* ok, cudaStream_t s) {
     if (c->fx_fit < 0) {
         TRY(ensure_small(c, 0, 0, 64));
         double v[3];
@@ -436,7 +439,7 @@ int fx_usable(ov_ctx* c, bool* ok, cudaStream_t s) {
         // (comparisons with a NaN are false)
         c->fx_fit = std::isfinite(v[0]) && v[0] > 0.0 && v[1] >= v[0] / 16.0 && v[2] >= 0.25 * std::sqrt(v[0]);
     }
-    *ok = c->fx_fit == 1;
+    *ok = c->fx_fit == 1 && (c->fx_no_room == 0 || nvec < c->fx_no_room);
     return OV_OK;
 }
 
@@ -474,6 +477,27 @@ int fx_links(ov_ctx* c, const SysSet& S, double scale2, FxLinks* L, cudaStream_t
     CKL();
     L->xlinks = ux;
     L->xidx = c->d_fxidx;
+    return OV_OK;
+}
+
+// The links of an FP64 recurrence in fixed point and its named vectors, nvec systems each.  Fixed point takes
+// more memory than FP64 (links of 576 B a site, 144 B a site and phase, one more vector a system): where the device
+// does not have it, what was taken is given back, *fx becomes false and the recurrence runs in FP64, for this many
+// systems until the next gauge field.
+int fx_prepare(ov_ctx* c, const SysSet& S, double scale2, std::initializer_list<std::pair<const char*, void**>> vectors,
+               long long nvec, FxLinks* L, bool* fx, cudaStream_t s) {
+    int rc = fx_links(c, S, scale2, L, s);
+    for (const auto& v : vectors)
+        if (rc == OV_OK) rc = workspace_fx(c, v.first, nvec, v.second);
+    if (rc != OV_ERR_OOM) return rc;
+    for (const auto& v : vectors) TRY(release_workspaces(c, std::string(v.first) + "/fx", s));
+    TRY(release_workspaces(c, "fx_Ux", s));
+    if (c->Ufx) CK(cudaFree(c->Ufx));
+    c->Ufx = nullptr;
+    c->fx_scale2 = 0.0;
+    c->fx_no_room = nvec;
+    *L = FxLinks();
+    *fx = false;
     return OV_OK;
 }
 
@@ -626,19 +650,18 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
     const double* d_phase = any_phase(S) ? c->d_phase : nullptr;
 
     bool fx = false;  // FP64: the recurrence on fixed-point vectors
-    if (std::is_same<ST, double>::value) TRY(fx_usable(c, &fx, s));
+    if (std::is_same<ST, double>::value) TRY(fx_usable(c, ns, &fx, s));
     void *xg, *xperp, *ys, *t, *bA, *bB;
     TRY(workspace(c, "sp_xg", prec, ns, &xg));
     TRY(workspace(c, "sp_xperp", prec, ns, &xperp));
     TRY(workspace(c, "sp_ys", prec, ns, &ys));
     void *xs = xperp, *p32 = nullptr;  // x_perp in the recurrence's storage; FP32 copy of its result
     FxLinks fxl;
-    if (fx) {
-        TRY(workspace_fx(c, "sp_t", ns, &t));
-        TRY(workspace_fx(c, "sp_bA", ns, &bA));
-        TRY(workspace_fx(c, "sp_bB", ns, &bB));
-        TRY(workspace_fx(c, "sp_xs", ns, &xs));
-    } else {
+    const double eps = c->p.eps, h = c->hw_norm;
+    const double alpha = 4.0 / ((1.0 - eps) * h * h);  // of the recurrence below
+    if (fx) TRY(fx_prepare(c, S, alpha, {{"sp_t", &t}, {"sp_bA", &bA}, {"sp_bB", &bB}, {"sp_xs", &xs}}, ns, &fxl, &fx, s));
+    if (!fx) {
+        xs = xperp;
         TRY(workspace(c, "sp_t", precs, ns, &t));
         TRY(workspace(c, "sp_bA", precs, ns, &bA));
         TRY(workspace(c, "sp_bB", precs, ns, &bB));
@@ -685,13 +708,10 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
     //   p = c_0 x_perp + Y b_1 - b_2.
     const int n = degree > 0 ? degree : c->p.poly_degree;
     const std::vector<double>& cf = coeffs_of(c, n);
-    const double eps = c->p.eps, h = c->hw_norm;
-    const double alpha = 4.0 / ((1.0 - eps) * h * h);
     const double beta = -2.0 * (1.0 + eps) / (1.0 - eps);
     const double m0 = c->p.m0;
     const void* U = links_of<R>(c);
     const void* Us = links_of<ST>(c);
-    if (fx) TRY(fx_links(c, S, alpha, &fxl, s));
     // algorithmic bytes per site of one launch: links once (shared by the systems) plus each
     // system's input, output and epilogue vectors
     const double Vd = (double)V, lb = site_link_bytes(precs), sb = fx ? 196 : site_spinor_bytes(precs);
@@ -1022,23 +1042,20 @@ int cheb_filter(ov_ctx* c, void* W, int m, double a, int degree, const SysSet& S
     const int prec = prec_of<R>();
     const size_t vb = vec_bytes(c, prec);
     bool fx = false;
-    if (std::is_same<R, double>::value) TRY(fx_usable(c, &fx, s));
-    const int cw = eig_chunk(c, prec, m, fx);
+    if (std::is_same<R, double>::value) TRY(fx_usable(c, eig_chunk(c, prec, m, true), &fx, s));
+    const double h = c->hw_norm, m0 = c->p.m0;
+    const double za = 2.0 / ((1.0 - a) * h * h), zb = -(1.0 + a) / (1.0 - a);
     void *Tm, *Tc, *tt;
     FxLinks fxl;
-    if (fx) {
-        TRY(workspace_fx(c, "flt_Tm", cw, &Tm));
-        TRY(workspace_fx(c, "flt_Tc", cw, &Tc));
-        TRY(workspace_fx(c, "flt_t", cw, &tt));
-    } else {
+    int cw = eig_chunk(c, prec, m, fx);
+    if (fx) TRY(fx_prepare(c, S, 2.0 * za, {{"flt_Tm", &Tm}, {"flt_Tc", &Tc}, {"flt_t", &tt}}, cw, &fxl, &fx, s));
+    if (!fx) {
+        cw = eig_chunk(c, prec, m);
         TRY(workspace(c, "flt_Tm", prec, cw, &Tm));
         TRY(workspace(c, "flt_Tc", prec, cw, &Tc));
         TRY(workspace(c, "flt_t", prec, cw, &tt));
     }
-    const double h = c->hw_norm, m0 = c->p.m0;
-    const double za = 2.0 / ((1.0 - a) * h * h), zb = -(1.0 + a) / (1.0 - a);
     const void* U = std::is_same<R, double>::value ? c->U64 : c->U32;
-    if (fx) TRY(fx_links(c, S, 2.0 * za, &fxl, s));
     for (int j0 = 0; j0 < m; j0 += cw) {
         const int nj = std::min(cw, m - j0);
         auto step = [&](const void* in, void* out, const Epilogue& e, bool half = false) {
@@ -1350,6 +1367,7 @@ int ov_set_gauge(ov_ctx* c, const void* U, int dtype, ov_stream_t stream) {
     launch_pack_gauge<double>(U, dtype, c->U64, c->g, s);
     c->fx_scale2 = 0.0;
     c->fx_fit = -1;
+    c->fx_no_room = 0;
     launch_pack_gauge<float>(U, dtype, c->U32, c->g, s);
     if (c->p.precision == OV_PREC_F16) launch_pack_gauge_half<H16>(U, dtype, c->U16, c->g.V, s);
     if (c->p.precision == OV_PREC_BF16) launch_pack_gauge_half<B16>(U, dtype, c->U16, c->g.V, s);
@@ -3096,25 +3114,19 @@ int tangent_poly_f64(ov_ctx* c, const void* X, const SysSet& S, void* Y, cudaStr
 
 // The same on fixed-point vectors where the links allow it.
 int tangent_poly(ov_ctx* c, const void* X, const SysSet& S, void* Y, cudaStream_t s) {
-    bool fx = false;
-    TRY(fx_usable(c, &fx, s));
-    if (!fx) return tangent_poly_f64(c, X, S, Y, s);
     const int ns = S.n;
-    void *x, *bA, *bB, *dA, *dB, *t, *u, *sv;
-    TRY(workspace_fx(c, "tg_x", ns, &x));
-    TRY(workspace_fx(c, "tg_bA", ns, &bA));
-    TRY(workspace_fx(c, "tg_bB", ns, &bB));
-    TRY(workspace_fx(c, "tg_dA", ns, &dA));
-    TRY(workspace_fx(c, "tg_dB", ns, &dB));
-    TRY(workspace_fx(c, "tg_t", ns, &t));
-    TRY(workspace_fx(c, "tg_u", ns, &u));
-    TRY(workspace_fx(c, "tg_s", ns, &sv));
     const int n = c->p.poly_degree;
     const double eps = c->p.eps, h = c->hw_norm;
     const double alpha = 4.0 / ((1.0 - eps) * h * h);
     const double beta = -2.0 * (1.0 + eps) / (1.0 - eps);
+    bool fx = false;
+    TRY(fx_usable(c, ns, &fx, s));
+    void *x, *bA, *bB, *dA, *dB, *t, *u, *sv;
     FxLinks L;  // of g H, g^2 = alpha: t = g H b1, u = g dH b1, s = g (H db1 + dH b1), then u = g dH t
-    TRY(fx_links(c, S, alpha, &L, s));
+    if (fx)
+        TRY(fx_prepare(c, S, alpha, {{"tg_x", &x}, {"tg_bA", &bA}, {"tg_bB", &bB}, {"tg_dA", &dA}, {"tg_dB", &dB}, {"tg_t", &t},
+                                     {"tg_u", &u}, {"tg_s", &sv}}, ns, &L, &fx, s));
+    if (!fx) return tangent_poly_f64(c, X, S, Y, s);
     launch_fx_from_f64(X, x, c->g.V, ns, 1.0, s);
     launch_fx_from_f64(X, bA, c->g.V, ns, c->coeffs[n], s);
     launch_fx_from_f64(X, dA, c->g.V, ns, 0.0, s);
