@@ -7,7 +7,6 @@ Tolerance: a thread's sum of at most some 100 products and the tree above it, 12
 products' magnitudes.  FP32: a product's own two roundings, 2 x 2^-24 of its magnitude at most; the sums keep
 what they round off, so the bound does not grow with the terms.
 """
-import os
 import subprocess
 
 import numpy as np
@@ -71,14 +70,8 @@ int main(int argc, char** argv) {
 
 
 @pytest.fixture(scope="module")
-def run32(tmp_path_factory):
-    from paper_1111_6288_gb300 import build
-
-    where = tmp_path_factory.mktemp("dots")
-    src, exe = where / "dots.cu", where / "dots"
-    src.write_text(PROGRAM)
-    subprocess.run([build.nvcc(), build.ARCH, "-std=c++17", "-I", build.CSRC, "-I", os.path.join(build.ROOT, "include"),
-                    str(src), build.LIB, "-Xlinker", "-rpath=" + os.path.dirname(build.LIB), "-o", str(exe)], check=True)
+def run32(cuda_program, tmp_path_factory):
+    exe, where = cuda_program(PROGRAM), tmp_path_factory.mktemp("dots")
 
     def run(a, b):
         for name, v in (("a", a), ("b", b)):
