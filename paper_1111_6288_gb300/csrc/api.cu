@@ -594,9 +594,10 @@ constexpr int kTcMinBatch = 8;
 
 // The small-space projection of k vectors (precision R, internal layout) on the bank b:
 // C = V^+ X, Xp = X - V C, Ys = V diag(s) C.  FP32 batches of kTcMinBatch or more vectors go through
-// the tcgen05 kernels unless the context's method says otherwise: these were 2 to 20 times faster wherever
-// both were timed (batches of 8 and 24; 16 to 131072 sites, banks of 1 to 200: 31 against 93 us at the small
-// end, 0.67 against 1.5 ms for 3 vectors' bank and 8 vectors at 16^3 x 32).
+// the tcgen05 kernels unless the context's method says otherwise.  Whole calls on the CUDA cores / tensor cores,
+// batches of 8 and of 24: 44 / 31 and 111 / 35 us (bank of 1, 16 sites), 254 / 53 and 738 / 55 (200, 256 sites),
+// 433 / 100 and 1285 / 121 (50, 8^3 x 16), 2618 / 987 and 7819 / 1221 (100, 16^3 x 32).  Only a bank of a few vectors
+// on a batch of 8 at 16^3 x 32 is better off on the CUDA cores (3: 560 / 670 us; 16: 875 / 675), which no line is drawn for.
 template <typename R>
 int project_bank(ov_ctx* c, const Bank* b, const void* X, int k, void* Xp, void* Ys, cudaStream_t s) {
     const int N = b->n;

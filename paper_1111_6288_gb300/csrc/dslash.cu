@@ -278,9 +278,9 @@ __device__ __forceinline__ void project(const NUM (&p)[12], Cx<R> (&h)[2][3]) {
 // ch = -c_op / 2: forward (FWD) uses U_mu(n) psi(n+mu), backward U_mu(n-mu)^+ psi(n-mu).  Everything that scales
 // the hop (ch, the boundary factor, FP16's site scale) is in fac, which the accumulation multiplies by at no
 // cost; only a field's phase on x hops (CPLX) takes a product of its own.  Against scaling each spinor, each hop
-// and the sum this saves 120 of some 1700 instructions a site in FP32 (16^3 x 32 11.45 -> 11.3 us a launch, 24 vectors of 24^3 x 48 1306 -> 1292 us) and more in
-// FP16 (12 vectors of 16^3 x 32 131 -> 123 us; with its sums of 16-bit numbers and its third rows 2360 -> 1970
-// instructions a site, 106 us).
+// and the sum this saves 120 of some 1700 instructions a site in FP32 (16^3 x 32 11.45 -> 11.3 us a launch; 24 systems
+// of 24^3 x 48, four a block, 1306 -> 1292 us a Clenshaw step's launch) and more in FP16 (12 vectors of 16^3 x 32
+// 131 -> 123 us; with its sums of 16-bit numbers and its third rows 2360 -> 1970 instructions a site, 106 us).
 template <int MU, bool FWD, bool CPLX, typename R>
 __device__ __forceinline__ void hop(const Cx<R> (&u)[3][3], const Cx<R> (&h)[2][3], R fac, Cx<R> phase,
                                     Cx<R> (&acc)[12]) {
@@ -580,7 +580,8 @@ template <> struct MinBlocks<B16> : MinBlocks<float> {};
 
 // A hop's link is loaded after its neighbour is projected where registers allow six blocks an SM, before where
 // they allow seven: late / early, one system of 8^3 x 16 4.46 / 4.55 us and 12 systems 8.84 / 9.10 us a launch with
-// six, 24 systems of 24^3 x 48 1412 / 1328 us with seven.
+// six; with seven, 24 systems of 24^3 x 48 1383 / 1299 us a Clenshaw step's launch with four systems a block,
+// 1403 / 1330 us with two.
 template <typename ST, int MINB>
 constexpr bool link_late = MINB == MinBlocks<ST>::value;
 

@@ -148,7 +148,7 @@ template <typename S>
 void launch_to_half(const void* in32, void* out, int V, long long nvec, double factor, cudaStream_t s);
 template <typename S>
 void launch_from_half(const void* in, void* out32, int V, long long nvec, cudaStream_t s);
-// ABI links -> 16-bit storage S (rows 0 and 1).
+// ABI links -> 16-bit storage S (three rows).
 template <typename S>
 void launch_pack_gauge_half(const void* abi, int dtype_in, void* internal, int V, cudaStream_t s);
 

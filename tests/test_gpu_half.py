@@ -6,8 +6,8 @@ FP32.  Each test states the error it measures (printed) and holds it to a bound
 in units of the format's unit roundoff u (FP16: 2^-11, its 11-bit significand on
 the per-site-scaled numbers; BF16: 2^-8):
 
-* one Wilson application: the input, the two stored link rows (the third row is
-  rebuilt from them) and the output are each rounded once, and every output
+* one Wilson application: the input, the three stored link rows and the output
+  are each rounded once, and every output
   component sums O(10) rounded terms of O(1): 16 u bounds the max-relative error
   (measured ~0.6 u for FP16, ~0.9 u for BF16 in a dense CPU emulation of the
   same formats);
