@@ -428,7 +428,12 @@ bool any_phase(const SysSet& S) {
 // test: two applications bring each spin to each other with coefficients of order 1.  Fields that do not mix colours so
 // (free, Abelian, nearly so), links of very different sizes and links that are not finite keep the FP64 stencil, five
 // times slower and exact to the last component.
-int fx_usable(ov_ctx* c, long long nvec, bool* ok, cudaStream_t s) {
+//
+// Coefficients that are not finite, and an operator's scale2 at the ends of FP64's range, keep the FP64 stencil too.
+int fx_usable(ov_ctx* c, long long nvec, double scale2, const double* coeffs, int ncoeffs, bool* ok, cudaStream_t s) {
+    *ok = scale2 > 1e-200 && scale2 < 1e200;
+    for (int k = 0; *ok && k < ncoeffs; ++k) *ok = std::isfinite(coeffs[k]);
+    if (!*ok) return OV_OK;
     if (c->fx_fit < 0) {
         TRY(ensure_small(c, 0, 0, 64));
         double v[3];
@@ -650,16 +655,18 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
     TRY(upload_sys(c, S, s));
     const double* d_phase = any_phase(S) ? c->d_phase : nullptr;
 
+    const int n = degree > 0 ? degree : c->p.poly_degree;
+    const std::vector<double>& cf = coeffs_of(c, n);
+    const double eps = c->p.eps, h = c->hw_norm;
+    const double alpha = 4.0 / ((1.0 - eps) * h * h);  // of the recurrence below
     bool fx = false;  // FP64: the recurrence on fixed-point vectors
-    if (std::is_same<ST, double>::value) TRY(fx_usable(c, ns, &fx, s));
+    if (std::is_same<ST, double>::value) TRY(fx_usable(c, ns, alpha, cf.data(), n + 1, &fx, s));
     void *xg, *xperp, *ys, *t, *bA, *bB;
     TRY(workspace(c, "sp_xg", prec, ns, &xg));
     TRY(workspace(c, "sp_xperp", prec, ns, &xperp));
     TRY(workspace(c, "sp_ys", prec, ns, &ys));
     void *xs = xperp, *p32 = nullptr;  // x_perp in the recurrence's storage; FP32 copy of its result
     FxLinks fxl;
-    const double eps = c->p.eps, h = c->hw_norm;
-    const double alpha = 4.0 / ((1.0 - eps) * h * h);  // of the recurrence below
     if (fx) TRY(fx_prepare(c, S, alpha, {{"sp_t", &t}, {"sp_bA", &bA}, {"sp_bB", &bB}, {"sp_xs", &xs}}, ns, &fxl, &fx, s));
     if (!fx) {
         xs = xperp;
@@ -707,8 +714,6 @@ int sign_pipeline(ov_ctx* c, const void* X, const SysSet& S, bool g5_in, Epilogu
     // Y = (2 Q^2 - (1 + eps))/(1 - eps) = alpha H_w^2 + beta/2:
     //   b_n = c_n x_perp;  b_k = c_k x_perp + 2 Y b_{k+1} - b_{k+2};
     //   p = c_0 x_perp + Y b_1 - b_2.
-    const int n = degree > 0 ? degree : c->p.poly_degree;
-    const std::vector<double>& cf = coeffs_of(c, n);
     const double beta = -2.0 * (1.0 + eps) / (1.0 - eps);
     const double m0 = c->p.m0;
     const void* U = links_of<R>(c);
@@ -1043,9 +1048,9 @@ int cheb_filter(ov_ctx* c, void* W, int m, double a, int degree, const SysSet& S
     const int prec = prec_of<R>();
     const size_t vb = vec_bytes(c, prec);
     bool fx = false;
-    if (std::is_same<R, double>::value) TRY(fx_usable(c, eig_chunk(c, prec, m, true), &fx, s));
     const double h = c->hw_norm, m0 = c->p.m0;
     const double za = 2.0 / ((1.0 - a) * h * h), zb = -(1.0 + a) / (1.0 - a);
+    if (std::is_same<R, double>::value) TRY(fx_usable(c, eig_chunk(c, prec, m, true), 2.0 * za, &zb, 1, &fx, s));
     void *Tm, *Tc, *tt;
     FxLinks fxl;
     int cw = eig_chunk(c, prec, m, fx);
@@ -3121,7 +3126,7 @@ int tangent_poly(ov_ctx* c, const void* X, const SysSet& S, void* Y, cudaStream_
     const double alpha = 4.0 / ((1.0 - eps) * h * h);
     const double beta = -2.0 * (1.0 + eps) / (1.0 - eps);
     bool fx = false;
-    TRY(fx_usable(c, ns, &fx, s));
+    TRY(fx_usable(c, ns, alpha, c->coeffs.data(), n + 1, &fx, s));
     void *x, *bA, *bB, *dA, *dB, *t, *u, *sv;
     FxLinks L;  // of g H, g^2 = alpha: t = g H b1, u = g dH b1, s = g (H db1 + dH b1), then u = g dH t
     if (fx)

@@ -546,13 +546,14 @@ __global__ void __launch_bounds__(128) fx_to_f64_k(const char* __restrict__ in, 
     }
 }
 
+// A coefficient of zero has an exponent below every other, so that its term sets no unit for the sum.
 fx::Coef make_coef(double c) {
     fx::Coef o{{0, 0}, 0, 0};
     if (c == 1.0 || c == -1.0) o.unit = (int)c;
     int k = 0;
     const double f = std::frexp(c, &k);  // c = f 2^k, 1/2 <= |f| < 1
     o.m = fx::split(std::llrint(std::ldexp(f, fx::kBits + 2)));
-    o.e = c == 0.0 ? 0 : k - 2;
+    o.e = c == 0.0 ? -(1 << 22) : k - 2;
     return o;
 }
 

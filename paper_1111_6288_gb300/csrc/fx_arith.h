@@ -97,7 +97,7 @@ FX_FN int bit_length(uint64_t v) {
 }
 
 // A real coefficient: value (hi 2^28 + lo) 2^(e - 56), |hi 2^28 + lo| < 2^59.  unit: +1 or -1 where
-// the coefficient is exactly that (no multiplication), else 0.
+// the coefficient is exactly that (no multiplication), else 0.  Finite coefficients only.
 struct Coef {
     Num m;
     int e;

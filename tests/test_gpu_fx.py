@@ -292,3 +292,57 @@ def test_only_shapes_that_differ_are_timed(P, dims, nrhs, shapes):
     P.apply_sign_Hw(ctx, x, x.clone())
     assert [int(k) for k in re.findall(r"(\d+)d?t?:", ctx.tune_info)] == shapes
     ctx.close()
+
+
+@pytest.mark.parametrize("coeffs, hw", [([0.0, 0.0, 0.0, 0.0, 1e-12], 6.5), ([1e-12, 0.0, 1e-12, 0.0, 0.0], 6.5),
+                                        ([0.0] * 5, 6.5), ([1.0, 0.5, 0.0, -0.25, 1e-30], 6.5),
+                                        ([1.0, 0.5, 0.25, 0.125, 0.0625], 1e200)])
+@pytest.mark.parametrize("op", ["sign", "derivative"])
+def test_the_callers_coefficients(P, coeffs, hw, op):
+    """Zeros among coefficients far below 1 set no unit; an operator's scale that underflows is FP64's.  The result is
+    off by the bound times the largest coefficient (and the growth of T_4 below the interval).  The derivative, whose
+    exact value is not at hand, scales with its coefficients by a power of two: to the last bit, but for a coefficient
+    of 1, which is added without a product in a finer unit (to the bound, n + 1 times over for the derivative's sum)."""
+    import torch
+
+    dims, bc, eps = (4, 3, 2, 5), (0, 0, 0, 1), 0.1
+    U = synth.random_su3_field(dims, 0.3, seed=43)
+    x = synth.gaussian_spinor(dims, 1, 44)
+
+    def run_with(cf):
+        ctx = P.Context(P.Params(dims=dims, bc=bc, m0=M0, hw_norm=hw, eps=eps, poly_degree=4, coeffs=cf, max_nrhs=1))
+        ctx.set_gauge(dev(U))
+        xd = dev(x)
+        y = torch.empty_like(xd)
+        if op == "sign":
+            P.apply_sign_Hw(ctx, xd, y)
+        else:
+            P.deflate(ctx, None, [], phase=0.3)
+            P.apply_dDdphi(ctx, xd, y, 0.0, phase=[0.3])
+        ctx.close()
+        return y.cpu().numpy()[0]
+
+    y = run_with(coeffs)
+    if op == "sign":
+        p = ov.OverlapParams(m0=M0, hw_norm=hw, eps=eps, degree=4, coeffs=np.array(coeffs), bc=(1.0, 1.0, 1.0, -1.0))
+        want = ov.sign_hw(U, x[0], p, ov.SmallSpace.empty(U.shape[1:5]), 0.0)
+        growth = np.cosh(4 * np.arccosh((1 + eps) / (1 - eps)))
+        assert np.linalg.norm(y - want) <= bound(4) * growth * np.abs(coeffs).max() * min(1.0, 6.5 / hw)
+    else:
+        scaled = run_with([c * 2.0**-100 for c in coeffs]) * 2.0**100
+        tol = 5 * bound(4) if 1.0 in coeffs else 0.0
+        assert np.linalg.norm(scaled - y) <= tol * np.linalg.norm(y)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_coefficients_that_are_not_finite(P, bad):
+    import torch
+
+    dims = (4, 3, 2, 5)
+    ctx = P.Context(P.Params(dims=dims, m0=M0, eps=0.1, poly_degree=2, coeffs=[1.0, bad, 0.5], max_nrhs=1))
+    ctx.set_gauge(dev(synth.random_su3_field(dims, 0.3, seed=45)))
+    x = dev(synth.gaussian_spinor(dims, 1, 46))
+    y = torch.zeros_like(x)
+    P.apply_sign_Hw(ctx, x, y)
+    ctx.close()
+    assert not np.isfinite(y.cpu().numpy()).any()
