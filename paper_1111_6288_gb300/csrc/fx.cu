@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(FX_THREADS, kBlocksPerSm) fx_dslash_kernel(con
                 int4* o = fx::at(a.out2 + off, s);
                 fx::store_spin(o, f, fu);
                 fx::store_spin(o, 3 - f, fl);
-                if (f == 0) *fx::exponent_at(a.out2 + off, s) = fx::bad_x(H) ? fx::kNanExp : ed;
+                if (f == 0) *fx::exponent_at(a.out2 + off, s) = H.bad_x ? fx::kNanExp : ed;
             }
         }
     }
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(FX_THREADS, kBlocksPerSm) fx_dslash_kernel(con
     fetch(std::integral_constant<int, 8>{});
     fx::mass_term(a, H, u, l);
     int E = H.eref - 1;
-    bool bad = H.bad;
+    bool bad = H.eref > fx::kNanTest;
     if constexpr (EPI) {
         const int ej = E + a.c0e;
         E = ej;
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(128) fx_split_kernel(const __grid_constant__ f
                 int4* o = fx::at(a.out2 + off, s);
                 fx::store_spin(o, f, fu);
                 fx::store_spin(o, 3 - f, fl);
-                if (f == 0) *fx::exponent_at(a.out2 + off, s) = fx::bad_x(H) ? fx::kNanExp : ed;
+                if (f == 0) *fx::exponent_at(a.out2 + off, s) = H.bad_x ? fx::kNanExp : ed;
             }
         }
         const i64 neg = k == 0 ? -(i64)f : 0;  // the y hops' lower spin; the z hops' has its sign already

@@ -224,10 +224,9 @@ FX_FN int normalise(i64 (&a)[6], i64 (&b)[6], uint64_t o, int e) {
 
 // The same for three of a site's numbers (0 and -1 are nothing here too).
 FX_FN int normalise(i64 (&a)[3], uint64_t o, int e) {
-    const int sh = bit_length(o) - kBits;
+    const int sh = o == 0 ? 1 : bit_length(o) - kBits;  // a shift by one bit makes 0 of both
     FX_UNROLL
-    for (int k = 0; k < 3; ++k)
-        a[k] = o == 0 ? 0 : sh > 0 ? shifted(a[k], sh, half_of(sh)) : (i64)((uint64_t)a[k] << -sh);
+    for (int k = 0; k < 3; ++k) a[k] = sh > 0 ? shifted(a[k], sh, half_of(sh)) : (i64)((uint64_t)a[k] << -sh);
     return o == 0 ? kZeroExp : e + sh;
 }
 
@@ -290,7 +289,8 @@ FX_FN void add_term(i64 (&a)[3], const int2 (&v)[3], int e, const Coef& c, int E
 // One lane's half of a site.  Hops are taken in the order y, z, t, x, forward before backward:
 // hop k goes in direction dir_of(k) to site nb[k].
 struct Half {
-    int f, x3, e0, eref, bad;
+    int f, x3, e0, eref;  // eref above kNanTest: the site or a neighbour holds a NaN
+    bool bad_x;           // an x neighbour does (the derivative has no other hops)
     int nb[8], ex[8];
     i64 up[6], own[6], oth[6];  // spin f, spin 2 + f, the other lane's lower spin
 };
@@ -322,7 +322,7 @@ FX_FN void half_setup(const Args& a, int s, int r, int f, Half& H) {
         eref = H.ex[k + 1] > eref ? H.ex[k + 1] : eref;
     }
     H.eref = eref;
-    H.bad = eref > kNanTest;
+    H.bad_x = H.ex[6] > kNanTest || H.ex[7] > kNanTest;
     FX_UNROLL
     for (int k = 0; k < 6; ++k) H.up[k] = H.own[k] = H.oth[k] = 0;
 }
@@ -364,9 +364,6 @@ FX_FN void half_hop(Half& H, const int4* pa, const int4* pb, const int4* u, i64 
         }
     }
 }
-
-// Whether an x hop brings a NaN (the derivative has no other hops).
-FX_FN bool bad_x(const Half& H) { return H.ex[6] > kNanTest || H.ex[7] > kNanTest; }
 
 // The x hops of DUAL: F + B into the sums, F - B (spins f and 3 - f) left in fu, fl; returns its exponent.
 FX_FN int dual_split(Half& H, i64 (&fu)[6], i64 (&fl)[6], const i64 (&bu)[6], const i64 (&bl)[6]) {
